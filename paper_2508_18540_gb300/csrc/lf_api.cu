@@ -155,18 +155,39 @@ size_t build_ws_layout(int64_t n, int32_t N, int32_t W, int32_t H, int64_t cap, 
     return w.bytes;
 }
 
-size_t comp_ws_layout(int32_t N, int32_t Vx, int32_t Vy, void* basev, CompWs* o)
+size_t comp_ws_layout(int32_t N, int32_t Vx, int32_t Vy, int VG, void* basev, CompWs* o)
 {
     char* base = static_cast<char*>(basev);
     size_t off = 0;
     CompWs w;
-    w.cx = carve<float>(base, off, (size_t)Vx * N * 3);
-    w.cy = carve<float>(base, off, (size_t)Vy * N * 3);
-    w.err = carve<int>(base, off, 1 + (size_t)N);
-    w.wide = w.err + 1;
+    w.err = carve<int>(base, off, 2);
+    w.np = base ? w.err + 1 : nullptr;
+    w.VG = VG;
+    const size_t groups = ((size_t)Vx + VG - 1) / VG, floats = VG == 1 ? 4 : 4 + 4 * (((size_t)VG + 3) / 4);
+    w.blk = carve<float>(base, off, groups * N * floats);
+    w.yt = carve<float2>(base, off, (size_t)Vy * N);
     w.bytes = align_up(off, 256);
     if (o) *o = w;
     return w.bytes;
+}
+
+// Size of a composite workspace: the tables of any view group width. The
+// limit of the static scratch is stated on the per-(view, plane) form, 12
+// bytes per (view column, plane) and (view row, plane); some width's tables
+// are no larger than that, up to their alignment.
+static size_t comp_ws_bytes(int32_t N, int32_t Vx, int32_t Vy)
+{
+    size_t most = 0;
+    for (int VG : {1, 3, 5, 9, 15}) {
+        const size_t b = comp_ws_layout(N, Vx, Vy, VG, nullptr, nullptr);
+        most = b > most ? b : most;
+    }
+    return most;
+}
+
+static size_t comp_static_bytes(int32_t N, int32_t Vx, int32_t Vy)
+{
+    return align_up(12 * (size_t)Vx * N, 256) + align_up(12 * (size_t)Vy * N, 256) + align_up(4 + 4 * (size_t)N, 256);
 }
 
 // stream each build workspace was last used on (for lf_mpi_status)
@@ -290,7 +311,7 @@ static void fill_comp_params(const lf_planes* planes, const lf_ref_camera* ref, 
 // argument checks shared by lf_composite and its adjoint; views_buf is the
 // output views (forward) or their gradient (backward)
 static lf_status check_composite_args(const lf_planes* planes, const lf_ref_camera* ref, const lf_view_set* views,
-                                      const float* views_buf, void* ws, size_t ws_bytes, CompWs* cw)
+                                      const float* views_buf, void* ws, size_t ws_bytes)
 {
     lf_status st = check_ref(ref);
     if (st != LF_OK) return st;
@@ -307,8 +328,6 @@ static lf_status check_composite_args(const lf_planes* planes, const lf_ref_came
     if (views->atlas_cols < 0) return fail(LF_ERR_INVALID_ARG, "atlas_cols must be >= 0");
     if (!ws) return fail(LF_ERR_WORKSPACE, "workspace is NULL");
     if (((uintptr_t)ws) % 256) return fail(LF_ERR_WORKSPACE, "workspace must be 256-byte aligned");
-    if (comp_ws_layout(planes->N, views->Vx, views->Vy, ws, cw) > ws_bytes)
-        return fail(LF_ERR_WORKSPACE, "composite workspace too small");
     return LF_OK;
 }
 
@@ -429,12 +448,16 @@ lf_status build_gaussians_prefix(const lf_gaussians* g, const lf_ref_camera* ref
 }
 
 lf_status composite_args(const lf_planes* planes, const lf_ref_camera* ref, const lf_view_set* views,
-                         const float* out, void* ws, size_t ws_bytes, CompWs* cw, CompParams* p)
+                         const float* out, void* ws, size_t ws_bytes, int VG, CompWs* cw, CompParams* p)
 {
-    const lf_status st = check_composite_args(planes, ref, views, out, ws, ws_bytes, cw);
+    const lf_status st = check_composite_args(planes, ref, views, out, ws, ws_bytes);
     if (st != LF_OK) return st;
     fill_comp_params(planes, ref, views, p);
-    return LF_OK;
+    if (comp_ws_layout(planes->N, views->Vx, views->Vy, VG ? VG : comp_views_fwd(*p), ws, cw) <= ws_bytes) return LF_OK;
+    // (the static scratch can be shorter than the widest tables: any width gives the same views)
+    for (int any : {15, 9, 5, 3, 1})
+        if (!VG && comp_ws_layout(planes->N, views->Vx, views->Vy, any, ws, cw) <= ws_bytes) return LF_OK;
+    return fail(LF_ERR_WORKSPACE, "composite workspace too small");
 }
 
 void raster_params(const lf_ref_camera* ref, int32_t N, int32_t dtype, RasterParams* p)
@@ -464,7 +487,7 @@ lf_status lf_composite_status(int32_t N, const lf_view_set* views, const void* c
 {
     if (!views || !cws || N < 1 || views->Vx < 1 || views->Vy < 1) return fail(LF_ERR_INVALID_ARG, "bad argument");
     CompWs cw;
-    comp_ws_layout(N, views->Vx, views->Vy, const_cast<void*>(cws), &cw);
+    comp_ws_layout(N, views->Vx, views->Vy, 1, const_cast<void*>(cws), &cw);   // the error word's place
     int err = 0;
     if (cudaStreamSynchronize(stream) != cudaSuccess ||
         cudaMemcpy(&err, cw.err, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess)
@@ -717,27 +740,32 @@ lf_status lf_filter_planes(const lf_planes* planes, double sigma, int32_t radius
 size_t lf_composite_workspace_size(int32_t N, const lf_view_set* views)
 {
     if (!views || N < 1 || views->Vx < 1 || views->Vy < 1) return 0;
-    return comp_ws_layout(N, views->Vx, views->Vy, nullptr, nullptr);
+    return comp_ws_bytes(N, views->Vx, views->Vy);
+}
+
+// coefficient tables, then the composite (state: its saving form)
+static lf_status run_composite(const lf_planes* planes, const CompWs& cw, const CompParams& p, float* out, float* state,
+                               cudaStream_t stream)
+{
+    lf_status st;
+    trace_begin("comp_coeffs", stream);
+    launch_comp_tables(p, planes->d, planes->count, cw, stream);
+    trace_end(stream);
+    if ((st = check_launch("composite coefficients")) != LF_OK) return st;
+    trace_begin(state ? "composite_save" : "composite", stream);
+    launch_composite(p, planes->rgba, cw, out, stream, reinterpret_cast<float4*>(state));
+    trace_end(stream);
+    return check_launch(state ? "composite (saving form)" : "composite");
 }
 
 lf_status lf_composite(const lf_planes* planes, const lf_ref_camera* ref, const lf_view_set* views, float* out,
                        void* ws, size_t ws_bytes, cudaStream_t stream)
 {
     CompWs cw;
-    lf_status st = check_composite_args(planes, ref, views, out, ws, ws_bytes, &cw);
-    if (st != LF_OK) return st;
     CompParams p;
-    fill_comp_params(planes, ref, views, &p);
-    if (cudaMemsetAsync(cw.err, 0, sizeof(int) * (1 + (size_t)planes->N), stream) != cudaSuccess)
-        return check_launch("composite reset");
-    trace_begin("comp_coeffs", stream);
-    launch_comp_coeffs(p, planes->d, planes->count, cw, stream);
-    trace_end(stream);
-    if ((st = check_launch("composite coefficients")) != LF_OK) return st;
-    trace_begin("composite", stream);
-    launch_composite(p, planes->rgba, planes->count, cw, out, stream);
-    trace_end(stream);
-    return check_launch("composite");
+    lf_status st = composite_args(planes, ref, views, out, ws, ws_bytes, 0, &cw, &p);
+    if (st != LF_OK) return st;
+    return run_composite(planes, cw, p, out, nullptr, stream);
 }
 
 size_t lf_composite_state_size(const lf_ref_camera* ref, const lf_view_set* views)
@@ -761,21 +789,11 @@ lf_status lf_composite_save(const lf_planes* planes, const lf_ref_camera* ref, c
                             float* state, size_t state_bytes, void* ws, size_t ws_bytes, cudaStream_t stream)
 {
     CompWs cw;
-    lf_status st = check_composite_args(planes, ref, views, out, ws, ws_bytes, &cw);
+    CompParams p;
+    lf_status st = composite_args(planes, ref, views, out, ws, ws_bytes, 0, &cw, &p);
     if (st != LF_OK) return st;
     if ((st = check_state(ref, views, state, state_bytes)) != LF_OK) return st;
-    CompParams p;
-    fill_comp_params(planes, ref, views, &p);
-    if (cudaMemsetAsync(cw.err, 0, sizeof(int) * (1 + (size_t)planes->N), stream) != cudaSuccess)
-        return check_launch("composite reset");
-    trace_begin("comp_coeffs", stream);
-    launch_comp_coeffs(p, planes->d, planes->count, cw, stream);
-    trace_end(stream);
-    if ((st = check_launch("composite coefficients")) != LF_OK) return st;
-    trace_begin("composite_save", stream);
-    launch_composite(p, planes->rgba, planes->count, cw, out, stream, reinterpret_cast<float4*>(state));
-    trace_end(stream);
-    return check_launch("composite (saving form)");
+    return run_composite(planes, cw, p, out, state, stream);
 }
 
 // state: NULL (two walks) or the saving forward's state
@@ -785,26 +803,24 @@ static lf_status composite_backward_impl(const lf_planes* planes, const lf_ref_c
                                          cudaStream_t stream)
 {
     CompWs cw;
-    lf_status st = check_composite_args(planes, ref, views, dviews, ws, ws_bytes, &cw);
+    CompParams p;
+    lf_status st = composite_args(planes, ref, views, dviews, ws, ws_bytes, 0, &cw, &p);
     if (st != LF_OK) return st;
     if (state && (st = check_state(ref, views, state, state_bytes)) != LF_OK) return st;
     if (!dplanes) return fail(LF_ERR_INVALID_ARG, "dplanes is NULL");
     if (views->atlas_cols > 0) return fail(LF_ERR_UNSUPPORTED, "the composite adjoint takes separate views only");
     if (((uintptr_t)dviews) % 16 || ((uintptr_t)dplanes) % 16)
         return fail(LF_ERR_INVALID_ARG, "dviews and dplanes must be 16-byte aligned");
-    CompParams p;
-    fill_comp_params(planes, ref, views, &p);
+    if (comp_ws_layout(planes->N, views->Vx, views->Vy, comp_views_bwd(p), ws, &cw) > ws_bytes)
+        return fail(LF_ERR_WORKSPACE, "composite workspace too small");
     const size_t dbytes = sizeof(float) * 4 * (size_t)planes->N * planes->W * planes->H;
-    if (cudaMemsetAsync(dplanes, 0, dbytes, stream) != cudaSuccess ||
-        cudaMemsetAsync(cw.err, 0, sizeof(int) * (1 + (size_t)planes->N), stream) != cudaSuccess)
-        return check_launch("composite backward reset");
+    if (cudaMemsetAsync(dplanes, 0, dbytes, stream) != cudaSuccess) return check_launch("composite backward reset");
     trace_begin("comp_coeffs", stream);
-    launch_comp_coeffs(p, planes->d, planes->count, cw, stream);
+    launch_comp_tables(p, planes->d, planes->count, cw, stream);
     trace_end(stream);
     if ((st = check_launch("composite coefficients")) != LF_OK) return st;
     trace_begin(state ? "composite_bwd_saved" : "composite_bwd", stream);
-    launch_composite_bwd(p, planes->rgba, planes->count, cw, dviews, dplanes, stream,
-                         reinterpret_cast<const float4*>(state));
+    launch_composite_bwd(p, planes->rgba, cw, dviews, dplanes, stream, reinterpret_cast<const float4*>(state));
     trace_end(stream);
     return check_launch("composite backward");
 }
@@ -925,7 +941,9 @@ lf_status lf_build_mpi_backward_voxels(const lf_voxels* v, const lf_ref_camera* 
 
 namespace lf {
 constexpr size_t kStaticCompBytes = 1u << 20;   // 1 MiB: e.g. N = 512 planes x 128 views
-static __device__ __align__(256) unsigned char g_comp_scratch[kStaticCompBytes];
+// the tables' alignment can take a few hundred bytes more than the size the limit is stated on
+constexpr size_t kStaticCompSlack = 4096;
+static __device__ __align__(256) unsigned char g_comp_scratch[kStaticCompBytes + kStaticCompSlack];
 
 // Device address of g_comp_scratch on the calling thread's current device.
 // In host code the array's name is only a host-side stand-in, so every call
@@ -955,7 +973,7 @@ lf_status lf_composite_noalloc(const lf_planes* planes, const lf_ref_camera* ref
     if (!planes || !views) return fail(LF_ERR_INVALID_ARG, "NULL argument");
     if (planes->N < 1 || views->Vx < 1 || views->Vy < 1 || views->Vx > 65535 || views->Vy > 65535)
         return fail(LF_ERR_INVALID_ARG, "N and view counts must be positive");
-    const size_t need = comp_ws_layout(planes->N, views->Vx, views->Vy, nullptr, nullptr);
+    const size_t need = comp_static_bytes(planes->N, views->Vx, views->Vy);
     if (need > lf::kStaticCompBytes)
         return fail(LF_ERR_WORKSPACE, "lf_composite_noalloc: N = " + std::to_string(planes->N) + " planes and " +
                                           std::to_string(views->Vx) + " x " + std::to_string(views->Vy) +
@@ -965,26 +983,16 @@ lf_status lf_composite_noalloc(const lf_planes* planes, const lf_ref_camera* ref
     lf_status st = lf::static_scratch(&scratch);
     if (st != LF_OK) return st;
     CompWs cw;
-    st = check_composite_args(planes, ref, views, out, scratch, lf::kStaticCompBytes, &cw);
-    if (st != LF_OK) return st;
     CompParams p;
-    fill_comp_params(planes, ref, views, &p);
-    if (cudaMemsetAsync(cw.err, 0, sizeof(int) * (1 + (size_t)planes->N), stream) != cudaSuccess)
-        return check_launch("composite reset");
-    trace_begin("comp_coeffs", stream);
-    launch_comp_coeffs(p, planes->d, planes->count, cw, stream);
-    trace_end(stream);
-    if ((st = check_launch("composite coefficients")) != LF_OK) return st;
-    trace_begin("composite", stream);
-    launch_composite(p, planes->rgba, planes->count, cw, out, stream);
-    trace_end(stream);
-    return check_launch("composite");
+    st = composite_args(planes, ref, views, out, scratch, lf::kStaticCompBytes + lf::kStaticCompSlack, 0, &cw, &p);
+    if (st != LF_OK) return st;
+    return run_composite(planes, cw, p, out, nullptr, stream);
 }
 
 lf_status lf_composite_noalloc_status(int32_t N, const lf_view_set* views, cudaStream_t stream)
 {
     if (!views || N < 1 || views->Vx < 1 || views->Vy < 1) return fail(LF_ERR_INVALID_ARG, "bad argument");
-    if (comp_ws_layout(N, views->Vx, views->Vy, nullptr, nullptr) > lf::kStaticCompBytes)
+    if (comp_static_bytes(N, views->Vx, views->Vy) > lf::kStaticCompBytes)
         return fail(LF_ERR_INVALID_ARG, "N and views exceed what lf_composite_noalloc accepts");
     void* scratch = nullptr;
     const lf_status st = lf::static_scratch(&scratch);

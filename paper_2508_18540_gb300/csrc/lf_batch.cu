@@ -24,16 +24,14 @@ struct lf_batch {
     int bilinear = 0;
     bool prepared = false;
     // device tables in the caller's batch workspace
-    unsigned long long* counters = nullptr;   // [2]: raster, composite item counters
     RasterScene* rtab = nullptr;
     CompScene* ctab = nullptr;
     // host copies (kept alive: the uploads read them)
     std::vector<RasterScene> rhost;
     std::vector<CompScene> chost;
     long long r_heavy = 0, r_total = 0, c_total = 0;   // raster grid: split-part CTAs, all CTAs
-    size_t max_stage = 0;
-    int maxN = 0;
-    int c_ctas = 0;
+    size_t c_smem = 0;                        // the largest composite layout
+    int tab_chunks = 0, tab_rows = 0;         // grid of the coefficient tables
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     long long graph_kernels = 0;              // kernels in one launch of the graph
@@ -73,6 +71,21 @@ bool plan_valid(const lf_batch_plan& pl)
            (pl.tile_x == 128 || pl.tile_x == 256 || pl.tile_x == 512) &&
            (pl.chunk_groups == 1 || pl.chunk_groups == 2 || pl.chunk_groups == kMaxChunkGroups) &&
            pl.schedule >= 0 && pl.schedule <= 2;
+}
+
+// Size limit of schedules 0 and 1: six stages of whole plane rows of a
+// tile_x x (256 / tile_x) tile and a table of maxN planes fit 200 KB. (The
+// composite itself stages only the windows that its tiles sample.)
+size_t batch_row_bytes(const CompParams& p, int tb, int tile_x)
+{
+    const int tx = std::min({(p.Nx + 31) / 32 * 32, tile_x, 256});
+    const size_t row = ((size_t)(16 + (p.W + 1) * tb) + 15) / 16 * 16;
+    return row * (size_t)(256 / tx) * (p.bilinear ? 2 : 1);
+}
+
+size_t batch_table_bytes(int maxN, int VG)
+{
+    return 96 + sizeof(float) * (size_t)maxN * (4 + 4 * ((VG + 3) / 4)) + sizeof(int) * (size_t)maxN;
 }
 
 lf_status check_scene(const lf_batch_scene& s, int i)
@@ -149,7 +162,6 @@ lf_status lf_batch_prepare(lf_batch* b, const lf_batch_plan* plan, void* ws, siz
     if (ws_bytes < batch_ws_bytes(b, groups))
         return fail(LF_ERR_WORKSPACE, "batch workspace too small for this plan (lf_batch_plan_workspace_size)");
     char* base = static_cast<char*>(ws);
-    b->counters = reinterpret_cast<unsigned long long*>(base);
     b->rtab = reinterpret_cast<RasterScene*>(base + align256(16));
     b->ctab = reinterpret_cast<CompScene*>(base + align256(16) + align256(sizeof(RasterScene) * n));
 
@@ -157,8 +169,8 @@ lf_status lf_batch_prepare(lf_batch* b, const lf_batch_plan* plan, void* ws, siz
     std::vector<RasterScene> r(n);
     std::vector<CompScene> c(n);
     std::vector<double> rwork(n), cwork(n);
-    size_t max_stage = 0;
-    int maxN = 0;
+    size_t row_bytes = 0, smem = 0;
+    int maxN = 0, tab_chunks = 0, tab_rows = 0;
     for (int i = 0; i < n; ++i) {
         lf_batch_scene& s = b->sc[i];
         const int64_t cap = ws_capacity(s.g.n, s.N, s.ref.W, s.ref.H, s.ws_bytes);
@@ -172,23 +184,29 @@ lf_status lf_batch_prepare(lf_batch* b, const lf_batch_plan* plan, void* ws, siz
 
         CompWs cw;
         CompParams cp;
-        const lf_status st = composite_args(&s.planes, &s.ref, &s.views, s.out, s.cws, s.cws_bytes, &cw, &cp);
+        const lf_status st = composite_args(&s.planes, &s.ref, &s.views, s.out, s.cws, s.cws_bytes,
+                                            pl.views_per_thread, &cw, &cp);
         if (st != LF_OK) return st;
         c[i].p = cp;
-        c[i].G = staged_geom(cp, tb, b->bilinear != 0, pl.views_per_thread, pl.tile_x);
+        c[i].G = comp_geom(cp, s.planes.rgba, pl.views_per_thread, false, false, pl.tile_x / 4);
         c[i].planes = static_cast<const char*>(s.planes.rgba);
+        c[i].d = s.planes.d;
         c[i].count = s.planes.count;
         c[i].w = cw;
         c[i].out = s.out;
-        c[i].nby = (cp.Ny + c[i].G.BY - 1) / c[i].G.BY;
-        c[i].nbz = (cp.Nx + c[i].G.TX - 1) / c[i].G.TX;
+        c[i].nbx = (cp.Nx + c[i].G.TX - 1) / c[i].G.TX;
         c[i].groups = groups;
         c[i].part = nullptr;
         cwork[i] = (double)cp.Vx * cp.Vy * cp.Nx * cp.Ny * cp.N;
-        max_stage = std::max(max_stage, c[i].G.stage_bytes);
+        row_bytes = std::max(row_bytes, batch_row_bytes(cp, tb, pl.tile_x));
         maxN = std::max(maxN, s.N);
+        smem = std::max(smem, (size_t)c[i].G.smem_bytes);
+        int chunks = 0, rows = 0;
+        comp_tables_grid(cp, pl.views_per_thread, &chunks, &rows);
+        tab_chunks = std::max(tab_chunks, chunks);
+        tab_rows = std::max(tab_rows, rows);
     }
-    if (pl.schedule != 2 && composite_batched_smem(max_stage, maxN, pl.views_per_thread) > 200 * 1024)
+    if (pl.schedule != 2 && 6 * row_bytes + batch_table_bytes(maxN, pl.views_per_thread) > 200 * 1024)
         return fail(LF_ERR_UNSUPPORTED, "lf_batch_prepare: the batch's largest plane row and N need more than "
                                         "200 KB of shared memory for the staged composite");
     // schedule: order of the scenes in the item tables
@@ -208,7 +226,7 @@ lf_status lf_batch_prepare(lf_batch* b, const lf_batch_plan* plan, void* ws, siz
         b->rhost[q] = R;
         CompScene C = c[co[q]];
         C.base = ct;
-        ct += (long long)C.G.groups_x * C.p.Vy * C.nby * C.nbz * C.groups;
+        ct += (long long)C.G.groups_x * C.p.Vy * ((C.p.Ny + C.G.BY - 1) / C.G.BY) * C.nbx * C.groups;
         b->chost[q] = C;
     }
     for (int q = 0; q < n; ++q) {
@@ -228,18 +246,10 @@ lf_status lf_batch_prepare(lf_batch* b, const lf_batch_plan* plan, void* ws, siz
             }
         }
     }
-    b->max_stage = max_stage;
-    b->maxN = maxN;
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) !=
-                                                  cudaSuccess)
-        return check_launch("device query");
-    const size_t smem = composite_batched_smem(max_stage, maxN, pl.views_per_thread);
-    // CTAs per SM: the composite's launch bounds aim at four (views per
-    // thread up to kTwoCtaViews) or two, as shared memory allows
-    int per_sm = pl.views_per_thread <= kTwoCtaViews ? 4 : 2;
-    while (per_sm > 1 && (size_t)per_sm * (smem + 1024) > (size_t)228 * 1024) --per_sm;
-    b->c_ctas = sms * per_sm;
+    if (ct > 0x7fffffffll) return fail(LF_ERR_UNSUPPORTED, "lf_batch_prepare: too many composite tiles");
+    b->c_smem = smem;
+    b->tab_chunks = tab_chunks;
+    b->tab_rows = tab_rows;
     if (cudaMemcpyAsync(b->rtab, b->rhost.data(), sizeof(RasterScene) * n, cudaMemcpyHostToDevice, stream) !=
             cudaSuccess ||
         cudaMemcpyAsync(b->ctab, b->chost.data(), sizeof(CompScene) * n, cudaMemcpyHostToDevice, stream) !=
@@ -274,8 +284,6 @@ lf_status lf_batch_render(lf_batch* b, cudaStream_t stream)
         }
         return LF_OK;
     }
-    if (cudaMemsetAsync(b->counters, 0, 2 * sizeof(unsigned long long), stream) != cudaSuccess)
-        return check_launch("batch counter reset");
     for (size_t i = 0; i < b->sc.size(); ++i) {
         lf_batch_scene& s = b->sc[i];
         BuildWs w;
@@ -291,24 +299,13 @@ lf_status lf_batch_render(lf_batch* b, cudaStream_t stream)
     trace_end(stream);
     if ((st = check_launch("batched raster")) != LF_OK) return st;
     trace_begin("comp_coeffs", stream);
-    for (size_t i = 0; i < b->sc.size(); ++i) {
-        lf_batch_scene& s = b->sc[i];
-        CompWs cw;
-        CompParams cp;
-        if ((st = composite_args(&s.planes, &s.ref, &s.views, s.out, s.cws, s.cws_bytes, &cw, &cp)) != LF_OK)
-            return st;
-        if (cudaMemsetAsync(cw.err, 0, sizeof(int) * (1 + (size_t)cp.N), stream) != cudaSuccess)
-            return check_launch("composite reset");
-        launch_comp_coeffs(cp, s.planes.d, s.planes.count, cw, stream);
-    }
+    launch_comp_tables_batched(b->ctab, (int)b->sc.size(), b->tab_chunks, b->tab_rows, stream);
     trace_end(stream);
     if ((st = check_launch("batched coefficients")) != LF_OK) return st;
     trace_begin("composite_batched", stream);
-    const bool ok = launch_composite_batched(b->ctab, (int)b->sc.size(), b->c_total, b->dtype, b->bilinear != 0,
-                                             b->plan.views_per_thread, b->max_stage, b->maxN, b->counters + 1,
-                                             b->c_ctas, stream);
+    launch_composite_batched(b->ctab, (int)b->sc.size(), b->c_total, b->dtype, b->bilinear != 0,
+                             b->plan.views_per_thread, b->c_smem, stream);
     trace_end(stream);
-    if (!ok) return fail(LF_ERR_UNSUPPORTED, "batched composite layout does not fit shared memory");
     if ((st = check_launch("batched composite")) != LF_OK) return st;
     if (b->plan.chunk_groups > 1) {
         trace_begin("merge_chunk_groups", stream);
@@ -446,7 +443,7 @@ lf_status lf_batch_status(lf_batch* b, cudaStream_t stream)
                                              std::to_string(h.total_dups) + " pairs, capacity " +
                                              std::to_string(h.dup_capacity));
         CompWs cw;
-        comp_ws_layout(b->sc[i].N, b->sc[i].views.Vx, b->sc[i].views.Vy, b->sc[i].cws, &cw);
+        comp_ws_layout(b->sc[i].N, b->sc[i].views.Vx, b->sc[i].views.Vy, 1, b->sc[i].cws, &cw);   // the error word's place
         if (cudaMemcpy(&err, cw.err, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess)
             return check_launch("error word read");
         if (err) return fail(LF_ERR_TIMEOUT, "batch scene " + std::to_string(i) + ": a composite wait gave up");

@@ -362,14 +362,18 @@ struct FilterParams {
 void launch_filter_planes(void* planes, int dtype, int N, int W, int H, const FilterParams& f, cudaStream_t s);
 
 // ---- composite ----------------------------------------------------------
+// Carved composite workspace: the error word first (its place depends on
+// nothing), then the tables of one launch (see lf_composite.cu).
 struct CompWs {
-    float* cx;      // [Vx][N][3] (gm, hn, hb) along x
-    float* cy;      // [Vy][N][3] along y
     int* err;       // [1] set to 1 if a bounded device wait gave up
-    int* wide;      // [N] 1 if some view's index range of plane k needs clamping
+    int* np;        // [1] non-empty planes
+    float* blk;     // [groups][N][CoefBlock] per-plane coefficients of every view group along x
+    float2* yt;     // [Vy][N] (gm, h) along y
+    int VG;         // views per group, and per thread of the composite kernels
     size_t bytes;
 };
-size_t comp_ws_layout(int32_t N, int32_t Vx, int32_t Vy, void* base, CompWs* out);
+// the tables for VG views per group
+size_t comp_ws_layout(int32_t N, int32_t Vx, int32_t Vy, int VG, void* base, CompWs* out);
 
 struct CompParams {
     int N, W, H, Nx, Ny, Vx, Vy, P_s, bilinear, dtype;
@@ -380,39 +384,36 @@ struct CompParams {
 };
 
 // staged composite layout (see lf_composite.cu)
-// Consumer threads of a staged-composite CTA (plus one producer warp): 256
-// for the forward kernels (two CTAs per SM at up to 15 views per thread,
-// four at 9 or fewer: an SM keeps working on one CTA's planes while the
-// other's warps wait at its ring), 512 for the adjoint (two CTAs per SM).
-constexpr int kStagedThreads = 256;
-constexpr int kBwdStagedThreads = 512;
-constexpr int kStages = 6;            // depth of its plane-row ring
-constexpr size_t kTwoCtaSmem = 112 * 1024;   // dynamic shared memory that still lets two CTAs share an SM
-constexpr int kTwoCtaViews = 9;               // widest view group run at the higher CTA count per SM
-struct StagedGeom {
-    int TX, BY, VG, rows_per_y;    // rows_per_y: 1 nearest, 2 bilinear
-    int padl;                      // zero texels left of every staged row (16 bytes)
-    int row_texels;                // padl + W + right pad, a multiple of 16 bytes
-    size_t row_bytes, stage_bytes, smem_bytes;
+constexpr int kCompThreads = 128;     // consumer threads of a CTA (plus one producer warp)
+constexpr int kStages = 4;            // most stages of its plane-row ring (two planes each)
+struct CompGeom {
+    int TX, BY, VG;                // tile columns, rows; views per thread
     int groups_x;                  // view groups per view row
-    int stages;                    // ring depth of the single-scene kernel (<= kStages)
-    size_t blend_bytes;            // bilinear: two FP32 row buffers per output row (single-scene kernel)
+    int stages;                    // ring depth (<= kStages)
+    int cap;                       // texels of a staged row window
+    bool bulk;                     // rows start on 16-byte boundaries (bulk copies)
+    uint32_t wcap;                 // texels of a warp's rows (bilinear, adjoint)
+    uint32_t hdr_bytes, win_bytes, plane_bytes, stage_bytes;   // a stage holds two planes
+    uint32_t rows_off, bar_off, stop_off, smem_bytes;   // offsets in shared memory, its size
 };
-StagedGeom staged_geom(const CompParams& p, int texel_bytes, bool bilinear, int VG, int tx_max,
-                       int threads = kStagedThreads);
+// tile_x: the most columns per tile (128, 64 or 32)
+CompGeom comp_geom(const CompParams& p, const void* planes, int VG, bool save, bool bwd, int tile_x);
+int comp_views_fwd(const CompParams& p);   // views per thread of the forward, of the adjoint
+int comp_views_bwd(const CompParams& p);
 
-// batched (several scenes, one persistent launch): per-scene item table;
+// batched (several scenes, one launch): per-scene item table;
 // item li of a scene: chunk group li % groups, then view group, then column
 // tile, then row band
 struct CompScene {
     CompParams p;
-    StagedGeom G;
+    CompGeom G;
     const char* planes;
+    const double* d;
     const int32_t* count;
     CompWs w;
     float* out;
     long long base;     // first global item of this scene
-    int nby, nbz;       // row bands, column tiles
+    int nbx;            // column tiles
     int groups;         // chunk groups: contiguous shares of the non-empty planes
     float4* part;       // groups > 1: [groups - 1][V][Ny][Nx] partial (Q, T) of groups 1.. (group 0 in out)
 };
@@ -420,23 +421,26 @@ constexpr int kMaxChunkGroups = 4;
 // groups > 1: composes the partials (group 0 in out, the others in part)
 // front to back into out's final views
 void launch_merge_chunk_groups(const CompParams& p, int groups, const float4* part, float* out, cudaStream_t s);
-void launch_comp_coeffs(const CompParams& p, const double* d, const int32_t* count, const CompWs& ws,
-                        cudaStream_t s);
-// smem_bytes: the largest staged layout of the batch (its stage size, N)
-bool launch_composite_batched(const CompScene* scenes_dev, int n_sc, long long total, int dtype, bool bilinear,
-                              int VG, size_t max_stage_bytes, int maxN, unsigned long long* counter, int n_ctas,
-                              cudaStream_t s);
-size_t composite_batched_smem(size_t max_stage_bytes, int maxN, int VG);
-// argument checks and parameters of one composite (lf_api.cu)
+// coefficient tables of one composite
+void launch_comp_tables(const CompParams& p, const double* d, const int32_t* count, const CompWs& ws, cudaStream_t s);
+// the same for every scene of a batch: the largest chunk and row counts that
+// comp_tables_grid gives for its scenes
+void comp_tables_grid(const CompParams& p, int VG, int* chunks, int* rows);
+void launch_comp_tables_batched(const CompScene* scenes_dev, int n_sc, int max_chunks, int max_rows, cudaStream_t s);
+// total: items of all scenes; smem: the largest layout of the batch
+void launch_composite_batched(const CompScene* scenes_dev, int n_sc, long long total, int dtype, bool bilinear,
+                              int VG, size_t smem, cudaStream_t s);
+// argument checks and parameters of one composite (lf_api.cu); VG 0: the forward's
+// choice of views per thread, or the one whose tables fit ws
 lf_status composite_args(const lf_planes* planes, const lf_ref_camera* ref, const lf_view_set* views,
-                         const float* out, void* ws, size_t ws_bytes, CompWs* cw, CompParams* p);
+                         const float* out, void* ws, size_t ws_bytes, int VG, CompWs* cw, CompParams* p);
 // state != null: the saving form, which also writes the adjoint's starting
 // state ([V][Ny][Nx] float4, separate views order)
-void launch_composite(const CompParams& p, const void* planes, const int32_t* count, const CompWs& ws,
-                      float* out, cudaStream_t s, float4* state = nullptr);
+void launch_composite(const CompParams& p, const void* planes, const CompWs& ws, float* out, cudaStream_t s,
+                      float4* state = nullptr);
 void launch_wait_selftest(unsigned long long limit_ns, int* result, cudaStream_t s);
 // state != null: start from the saving forward's state (one plane walk)
-void launch_composite_bwd(const CompParams& p, const void* planes, const int32_t* count, const CompWs& ws,
-                          const float* dviews, float* dplanes, cudaStream_t s, const float4* state = nullptr);
+void launch_composite_bwd(const CompParams& p, const void* planes, const CompWs& ws, const float* dviews,
+                          float* dplanes, cudaStream_t s, const float4* state = nullptr);
 
 }  // namespace lf
