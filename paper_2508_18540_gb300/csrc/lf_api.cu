@@ -110,11 +110,10 @@ size_t build_ws_layout(int64_t n, int32_t N, int32_t W, int32_t H, int64_t cap, 
     char* base = static_cast<char*>(basev);
     const long long supers = (long long)((W + kSuper - 1) / kSuper) * ((H + kSuper - 1) / kSuper);
     const long long S = supers * N;                                 // (super-tile, chunk) lists
-    const long long nmax = n > cap ? n : cap;
-    const long long nb = (nmax + kRadixBlockKeys - 1) / kRadixBlockKeys + 1;
-    const long long nbd = (n + kDupBlock - 1) / kDupBlock + 1;
     const size_t nn = (size_t)(n > 0 ? n : 1);
     const size_t cc = (size_t)(cap > 0 ? cap : 1);
+    const size_t kk = nn > cc ? nn : cc;                            // the depth sort uses the pair keys, too
+    const int tile_passes = tile_sort_passes(tile_bits_for(supers));
     size_t off = 0;
     BuildWs w;
     w.hdr = carve<WsHeader>(base, off, 1);
@@ -130,12 +129,23 @@ size_t build_ws_layout(int64_t n, int32_t N, int32_t W, int32_t H, int64_t cap, 
     w.r_rgb = carve<float4>(base, off, nn);
     w.r_den = carve<float4>(base, off, 2 * nn);
     w.r_chunk = carve<int32_t>(base, off, nn);
-    w.hist = carve<uint32_t>(base, off, (size_t)kSortDigits * nb);
-    w.dtot = carve<uint32_t>(base, off, (size_t)kSortDigits);
-    w.bsum = carve<uint32_t>(base, off, (size_t)nbd);
+    // 256-rank blocks while they make no more than one wave at four per SM
+    w.dup_block = nn <= 152 * 4 * 256 ? 256 : 1024;
+    const long long nbd = (n + w.dup_block - 1) / w.dup_block + 1;
+    // sweeps: over the primitives, and over their pairs (about two each)
+    w.kpt_depth = sweep_kpt((long long)nn);
+    w.kpt_tile = sweep_kpt(2 * (long long)nn);
+    w.nb_depth = ((long long)nn + kSweepThreads * w.kpt_depth - 1) / (kSweepThreads * w.kpt_depth);
+    w.nb_tile = ((long long)cc + kSweepThreads * w.kpt_tile - 1) / (kSweepThreads * w.kpt_tile);
+    w.dhist = carve<uint32_t>(base, off, (size_t)(kDepthPasses + kTilePassesMax) * kSortDigits);
+    const size_t zero_from = off - sizeof(uint32_t) * (size_t)(kDepthPasses + kTilePassesMax) * kSortDigits;
+    w.bstat = carve<unsigned long long>(base, off, (size_t)nbd);
+    w.sstat = carve<unsigned long long>(base, off,
+                                        (size_t)kSortDigits * (kDepthPasses * w.nb_depth + tile_passes * w.nb_tile));
+    w.zero_bytes = off - zero_from;
     w.chunk_start = carve<int32_t>(base, off, (size_t)N + 1);
-    w.tkeyA = carve<uint32_t>(base, off, cc);
-    w.tkeyB = carve<uint32_t>(base, off, cc);
+    w.tkeyA = carve<uint32_t>(base, off, kk);
+    w.tkeyB = carve<uint32_t>(base, off, kk);
     w.entA = carve<uint32_t>(base, off, cc);
     w.entB = carve<uint32_t>(base, off, cc);
     w.seg = carve<int2>(base, off, (size_t)S);
@@ -149,7 +159,6 @@ size_t build_ws_layout(int64_t n, int32_t N, int32_t W, int32_t H, int64_t cap, 
     w.r_arrive = carve<int>(base, off, (size_t)S);
     w.r_part = carve<float4>(base, off, (size_t)slots * kSuper * kSuper);
     w.bytes = align_up(off, 256);
-    w.nb_sort = nb;
     w.nb_dup = nbd;
     if (o) *o = w;
     return w.bytes;
@@ -383,10 +392,10 @@ static lf_status build_common(int64_t n, const lf_ref_camera* ref, int32_t N, in
     h.supers_x = (ref->W + kSuper - 1) / kSuper;
     h.supers_y = (ref->H + kSuper - 1) / kSuper;
     h.binning = binning;
-    // the header is written by a kernel so the whole build stays on the stream
-    launch_init_header(h, w.hdr, stream);
-    if ((st = check_launch("header init")) != LF_OK) return st;
     const long long n_supers = (long long)h.supers_x * h.supers_y;
+    // the header is written by a kernel so the whole build stays on the stream
+    launch_init(h, w, n_supers * N, stream);
+    if ((st = check_launch("header init")) != LF_OK) return st;
 
     ProjParams pp;
     fill_proj_params(ref, n, &pp);
@@ -408,12 +417,13 @@ static lf_status build_common(int64_t n, const lf_ref_camera* ref, int32_t N, in
                                  : static_cast<const lf_voxels*>(raster_arg)->rgb;
     const float* dens8 = kind == 0 ? nullptr : static_cast<const lf_voxels*>(raster_arg)->density8;
     trace_begin("bin", stream);
-    launch_bin(w, bp, n, out->chunk, out->d, out->count, out->rect, rgb, dens8, kind, stream);
+    launch_bin(w, bp, n, out->chunk, out->rect, rgb, dens8, kind, h.supers_x, (int)n_supers, stream);
     trace_end(stream);
     if ((st = check_launch("bin")) != LF_OK) return st;
 
     trace_begin("tile_lists", stream);
-    const uint32_t* ranks = launch_tile_lists(w, n, cap, N, h.supers_x, (int)n_supers, stream);
+    const uint32_t* ranks =
+        launch_tile_lists(w, bp, cap, h.supers_x, (int)n_supers, out->d, out->count, stream);
     trace_end(stream);
     if ((st = check_launch("tile lists")) != LF_OK) return st;
 
@@ -646,6 +656,7 @@ lf_status lf_mpi_status(const void* ws, int64_t* needed, int64_t* culled_in)
     if (cudaMemcpy(&h, ws, sizeof(h), cudaMemcpyDeviceToHost) != cudaSuccess) return check_launch("header read");
     if (needed) *needed = (int64_t)h.total_dups;
     if (culled_in) *culled_in = (int64_t)h.M;
+    if (h.timeout) return fail(LF_ERR_TIMEOUT, "a bounded wait of the build gave up");
     if (h.overflow)
         return fail(LF_ERR_OVERFLOW, "tile list needs " + std::to_string(h.total_dups) + " pairs, capacity " +
                                          std::to_string(h.dup_capacity));

@@ -438,6 +438,7 @@ lf_status lf_batch_status(lf_batch* b, cudaStream_t stream)
         int err = 0;
         if (cudaMemcpy(&h, b->sc[i].ws, sizeof(h), cudaMemcpyDeviceToHost) != cudaSuccess)
             return check_launch("header read");
+        if (h.timeout) return fail(LF_ERR_TIMEOUT, "batch scene " + std::to_string(i) + ": a build wait gave up");
         if (h.overflow)
             return fail(LF_ERR_OVERFLOW, "batch scene " + std::to_string(i) + ": tile list needs " +
                                              std::to_string(h.total_dups) + " pairs, capacity " +

@@ -19,9 +19,10 @@ constexpr int kTile = 16;                 // raster tile edge (pixels): one CTA 
 constexpr int kTilePix = kTile * kTile;
 constexpr int kSuper = 32;                // list super-tile edge (pixels): lists per (super-tile, chunk)
 constexpr int kTilesPerSuper = kSuper / kTile;
-constexpr int kRadixBlockKeys = 2048;     // keys per radix-sort block
 constexpr int kSortDigits = 256;          // 8-bit radix digits
-constexpr int kDupBlock = 1024;           // ranks per block of the tile-pair emission
+constexpr int kSweepThreads = 512;        // threads of a radix-sweep block
+constexpr int kDepthPasses = 3;           // digits of the truncated depth key
+constexpr int kTilePassesMax = 3;         // digits of a super-tile id (planes up to 32768^2)
 constexpr uint64_t kInvalidKey = ~0ull;
 
 // bytes of one RGBA texel of a plane type
@@ -144,6 +145,27 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity)
 
 #endif
 
+// ---- decoupled look-back ---------------------------------------------------
+// A block publishes its own sum (kSumOwn), then, once it has added up the
+// blocks before it, the sum up to and with itself (kSumAll), in one 64-bit
+// word: two flag bits over a 62-bit count.
+#ifdef __CUDACC__
+constexpr unsigned long long kSumOwn = 1ull << 62, kSumAll = 2ull << 62, kSumMask = kSumOwn - 1ull;
+constexpr int kLookbackTries = 1 << 20;   // polls without progress (about a second) before a block gives up
+
+__device__ __forceinline__ unsigned long long ld_word(const unsigned long long* p)
+{
+    unsigned long long v;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+
+__device__ __forceinline__ void st_word(unsigned long long* p, unsigned long long v)
+{
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+#endif
+
 // ---- RGBA8 unorm codec (exact, no conversion-unit instructions) -------------
 // decode: byte k of u placed under the exponent of 2^23 reads 2^23 + byte;
 //         subtracting 2^23 leaves the byte as an exact FP32 integer.
@@ -207,6 +229,10 @@ struct WsHeader {
     // split into parts
     unsigned int r_heavy;         // parts of split lists
     int r_seg;                    // entries per part (0x7fffffff: no list is split)
+    // blocks of the sweeps and of the binning take their place in order from
+    // these counters, so that a block only ever waits for running ones
+    unsigned int ticket[kDepthPasses + kTilePassesMax + 1];
+    int timeout;                  // a bounded wait of the build gave up
 };
 
 // Split lists of the Gaussian raster: a list of L > r_seg entries is cut into
@@ -232,9 +258,11 @@ struct BuildWs {
     float4* r_rgb;                // [n] colour
     float4* r_den;                // [2 n] voxel corner densities
     int32_t* r_chunk;             // [n]
-    uint32_t* hist;               // [kSortDigits * nb] radix histograms
-    uint32_t* dtot;               // [kSortDigits] per-digit totals of a radix pass
-    uint32_t* bsum;               // [nbd] block sums of the pair emission
+    // zeroed together by the build's first kernel, from dhist on
+    uint32_t* dhist;              // [kDepthPasses + kTilePassesMax][kSortDigits] digit totals of every pass
+    unsigned long long* bstat;    // [nb_dup] look-back words of the pair emission
+    unsigned long long* sstat;    // look-back words of the sweeps: per pass [blocks][kSortDigits]
+    size_t zero_bytes;            // from dhist to the end of sstat
     int32_t* chunk_start;         // [N + 1]
     uint32_t* tkeyA;              // [cap] tile id of every (tile, rank) pair
     uint32_t* tkeyB;
@@ -247,7 +275,10 @@ struct BuildWs {
     int* r_arrive;                // [lists] parts of a split list finished
     long long r_nslots;           // partial-result slots
     size_t bytes;
-    long long nb_sort, nb_dup;
+    long long nb_dup;
+    int dup_block;                // ranks per block of the binning and pair emission
+    int kpt_depth, kpt_tile;      // keys per thread of the sweeps
+    long long nb_depth, nb_tile;  // blocks of a sweep
 };
 
 size_t build_ws_layout(int64_t n, int32_t N, int32_t W, int32_t H, int64_t cap, void* base, BuildWs* out);
@@ -286,7 +317,9 @@ struct BinParams {
 };
 
 // ---- launchers ----------------------------------------------------------
-void launch_init_header(const WsHeader& h, WsHeader* d, cudaStream_t s);
+// writes the header, and zeroes the look-back words, digit totals and the n_lists
+// list ranges
+void launch_init(const WsHeader& h, const BuildWs& ws, long long n_lists, cudaStream_t s);
 void launch_project_gaussians(const lf_gaussians& g, const ProjParams& p, const BuildWs& ws, int32_t* rect,
                               int32_t* chunk, cudaStream_t s);
 void launch_project_voxels(const lf_voxels& v, const ProjParams& p, const BuildWs& ws, int32_t* rect,
@@ -297,15 +330,19 @@ void launch_project_voxels(const lf_voxels& v, const ProjParams& p, const BuildW
 // (IEEE bits, by primitive index). Uses tkeyA/tkeyB, valB, keyB as scratch.
 void sort_depth_keys(const BuildWs& ws, long long n, cudaStream_t s);
 
-void launch_bin(const BuildWs& ws, const BinParams& p, long long n, int32_t* chunk, double* d, int32_t* count,
-                const int32_t* rect, const float* rgb, const float* dens8, int kind, cudaStream_t s);
-// (super-tile, chunk) lists: (super-tile, rank) pairs emitted in rank order,
-// stable sort by super-tile, [start, end) of every (super-tile, chunk) list.
+// Chunk of every rank, rank-ordered copies, first rank of every chunk, and
+// the (super-tile, rank) pairs in rank order with their digit totals.
+void launch_bin(const BuildWs& ws, const BinParams& p, long long n, int32_t* chunk, const int32_t* rect,
+                const float* rgb, const float* dens8, int kind, int supers_x, int n_supers, cudaStream_t s);
+// (super-tile, chunk) lists: stable sort of the pairs by super-tile, [start,
+// end) of every (super-tile, chunk) list, and the plane distances and counts.
 // Returns the sorted ranks.
-const uint32_t* launch_tile_lists(const BuildWs& ws, long long n, long long cap, int N, int supers_x, int n_supers,
-                                  cudaStream_t s);
+const uint32_t* launch_tile_lists(const BuildWs& ws, const BinParams& p, long long cap, int supers_x, int n_supers,
+                                  double* d, int32_t* count, cudaStream_t s);
 void sort_tile_keys(const BuildWs& ws, long long cap, int tile_bits, cudaStream_t s, uint32_t** keys_out,
                     uint32_t** vals_out);
+// keys per thread of a sweep over about n keys
+int sweep_kpt(long long n);
 int tile_sort_passes(int tile_bits);
 int tile_bits_for(long long tiles);
 

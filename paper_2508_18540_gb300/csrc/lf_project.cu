@@ -13,16 +13,28 @@
 
 namespace lf {
 
-__global__ void k_init_header(WsHeader h, WsHeader* d)
+// The build's first kernel: the header, zeroed look-back words and digit
+// totals (16-byte words; a region's last words may be its alignment's), and
+// empty list ranges.
+__global__ void __launch_bounds__(256) k_init(WsHeader h, BuildWs w, long long n_lists)
 {
     pdl_wait();
     pdl_trigger();
-    *d = h;
+    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x, stride = (long long)gridDim.x * blockDim.x;
+    if (t == 0) *w.hdr = h;
+    const uint4 z = make_uint4(0u, 0u, 0u, 0u);
+    uint4* a = reinterpret_cast<uint4*>(w.dhist);
+    for (long long i = t; i < (long long)(w.zero_bytes / 16); i += stride) a[i] = z;
+    int2* seg = w.seg;
+    for (long long i = t; i < n_lists; i += stride) seg[i] = make_int2(0, 0);
 }
 
-void launch_init_header(const WsHeader& h, WsHeader* d, cudaStream_t s)
+void launch_init(const WsHeader& h, const BuildWs& ws, long long n_lists, cudaStream_t s)
 {
-    launch_pdl(k_init_header, dim3(1), dim3(1), 0, s, h, d);
+    const long long words = (long long)(ws.zero_bytes / 16) + n_lists;
+    long long blocks = (words + 1023) / 1024;
+    blocks = blocks < 1 ? 1 : blocks > 152 * 8 ? 152 * 8 : blocks;
+    launch_pdl(k_init, dim3((unsigned)blocks), dim3(256), 0, s, h, ws, n_lists);
     note_launches(1);
 }
 
@@ -47,7 +59,9 @@ __device__ __forceinline__ unsigned long long warp_max_u64(unsigned long long v)
 }
 
 constexpr int kProjThreads = 256;
-constexpr int kProjItems = 4;   // primitives per thread (block-strided)
+// primitives per thread (block-strided): 4 (one atomic of each kind per 1024
+// primitives), 1 while the blocks are fewer than the SMs can hold at once
+inline int proj_items(long long n) { return n <= 152ll * 4 * kProjThreads ? 1 : 4; }
 
 // Culled-in count and depth key range of the primitives one thread projected.
 struct KeyStats {
@@ -165,13 +179,13 @@ __device__ __forceinline__ bool gauss_footprint(const ProjParams& p, float m0, f
 }
 
 __global__ void __launch_bounds__(kProjThreads) k_project_gaussians(lf_gaussians g, ProjParams p, BuildWs w,
-                                                                    int4* rect_out, int32_t* chunk_out)
+                                                                    int4* rect_out, int32_t* chunk_out, int items)
 {
     pdl_wait();
     pdl_trigger();
     KeyStats st;
-    for (int it = 0; it < kProjItems; ++it) {
-        const long long i = ((long long)blockIdx.x * kProjItems + it) * kProjThreads + threadIdx.x;
+    for (int it = 0; it < items; ++it) {
+        const long long i = ((long long)blockIdx.x * items + it) * kProjThreads + threadIdx.x;
         unsigned long long key = kInvalidKey;
         if (i < p.n) {
             const float m0 = g.means[3 * i + 0], m1 = g.means[3 * i + 1], m2 = g.means[3 * i + 2];
@@ -194,7 +208,6 @@ __global__ void __launch_bounds__(kProjThreads) k_project_gaussians(lf_gaussians
             }
             rect_out[i] = rect;
             w.keyA[i] = key;
-            w.valA[i] = (uint32_t)i;
         }
         st.add(key);
     }
@@ -205,13 +218,13 @@ __global__ void __launch_bounds__(kProjThreads) k_project_gaussians(lf_gaussians
 // Depth = centre depth; culled unless the nearest corner lies past z_near;
 // footprint = bounding box of the 8 projected corners (pixel centres inside).
 __global__ void __launch_bounds__(kProjThreads) k_project_voxels(lf_voxels v, ProjParams p, BuildWs w,
-                                                                 int4* rect_out, int32_t* chunk_out)
+                                                                 int4* rect_out, int32_t* chunk_out, int items)
 {
     pdl_wait();
     pdl_trigger();
     KeyStats st;
-    for (int it = 0; it < kProjItems; ++it) {
-        const long long i = ((long long)blockIdx.x * kProjItems + it) * kProjThreads + threadIdx.x;
+    for (int it = 0; it < items; ++it) {
+        const long long i = ((long long)blockIdx.x * items + it) * kProjThreads + threadIdx.x;
         unsigned long long key = kInvalidKey;
         if (i < p.n) {
             double s = p.base_size;
@@ -268,7 +281,6 @@ __global__ void __launch_bounds__(kProjThreads) k_project_voxels(lf_voxels v, Pr
             }
             rect_out[i] = rect;
             w.keyA[i] = key;
-            w.valA[i] = (uint32_t)i;
         }
         st.add(key);
     }
@@ -445,9 +457,10 @@ void launch_project_gaussians(const lf_gaussians& g, const ProjParams& p, const 
                               int32_t* chunk, cudaStream_t s)
 {
     if (p.n <= 0) return;
-    const long long per = (long long)kProjThreads * kProjItems;
+    const int items = proj_items(p.n);
+    const long long per = (long long)kProjThreads * items;
     const unsigned blocks = (unsigned)((p.n + per - 1) / per);
-    launch_pdl(k_project_gaussians, dim3(blocks), dim3(kProjThreads), 0, s, g, p, ws, reinterpret_cast<int4*>(rect), chunk);
+    launch_pdl(k_project_gaussians, dim3(blocks), dim3(kProjThreads), 0, s, g, p, ws, reinterpret_cast<int4*>(rect), chunk, items);
     note_launches(1);
 }
 
@@ -455,9 +468,10 @@ void launch_project_voxels(const lf_voxels& v, const ProjParams& p, const BuildW
                            cudaStream_t s)
 {
     if (p.n <= 0) return;
-    const long long per = (long long)kProjThreads * kProjItems;
+    const int items = proj_items(p.n);
+    const long long per = (long long)kProjThreads * items;
     const unsigned blocks = (unsigned)((p.n + per - 1) / per);
-    launch_pdl(k_project_voxels, dim3(blocks), dim3(kProjThreads), 0, s, v, p, ws, reinterpret_cast<int4*>(rect), chunk);
+    launch_pdl(k_project_voxels, dim3(blocks), dim3(kProjThreads), 0, s, v, p, ws, reinterpret_cast<int4*>(rect), chunk, items);
     note_launches(1);
 }
 

@@ -10,24 +10,32 @@
 //    primitives in the first pass and sorts stably in three passes (the
 //    first pass takes each key's index as its value, so equal keys stay in
 //    index order). Keys that share the truncated value form runs that are
-//    then put in (full key, index) order: runs of up to 32 by one thread
-//    (insertion), longer runs by one CTA each (Batcher's odd-even merge
-//    network, in shared memory up to 2048 keys, in global memory beyond).
-//    The run pass keeps the order exact for any input; 24 bits trade a
-//    fourth pass for short runs (1M Gaussians over depths 1.5..10: runs of at
-//    most 5 keys, 12k pairs to reorder; grid-aligned voxels: runs of equal
-//    full keys, already in order).
-//  - the 3D tiling (Sec. 4.4): 32-bit keys = tile id of every (tile, rank)
-//    pair emitted in rank order; the stable sort groups the pairs by tile and
-//    keeps each tile's pairs in depth order.
+//    then put in (full key, index) order: every member of a run of up to 32
+//    counts the members before it, longer runs that are out of order go to
+//    one CTA each (Batcher's odd-even merge network, in shared memory up to
+//    2048 keys, in global memory beyond). The run pass keeps the order exact
+//    for any input; 24 bits trade a fourth pass for short runs (1M Gaussians
+//    over depths 1.5..10: runs of at most 5 keys, 12k pairs to reorder;
+//    grid-aligned voxels: runs of equal full keys, already in order).
+//  - the 3D tiling (Sec. 4.4): 32-bit keys = super-tile id of every
+//    (super-tile, rank) pair emitted in rank order; the stable sort groups the
+//    pairs by super-tile and keeps each one's pairs in depth order.
 //
-// Each pass is reduce-then-scan over blocks of 2048 keys:
-//   k_upsweep   per-block digit histogram (warp-aggregated shared atomics);
-//   k_rowscan   one CTA per digit scans that digit's per-block counts;
-//   k_downsweep ranks the block's keys stably (ballot-based digit matching,
-//               per-warp counters, warps own contiguous key ranges), exchanges
-//               them through shared memory into digit order and writes every
-//               digit run contiguously.
+// One kernel per pass (k_sweep), with the digit totals of all passes known
+// beforehand (k_depth_hist; the pair emission): a block of 512 threads ranks
+// its 2048 or 4096 keys stably (ballot-based digit matching, per-warp
+// counters, warps own contiguous key ranges), publishes its digit counts,
+// exchanges the keys through shared memory into digit order, adds up the
+// counts of the blocks before it by decoupled look-back (one thread per
+// digit, 16 predecessors per round trip), and writes every digit run
+// contiguously. Blocks of 2048 keys while those make one wave of the chip's
+// 152 SMs, else 4096 (two blocks of 64 registers a thread per SM; 8192 keys
+// at one block per SM left too few warps for the ranking: 33 us a pass at 1M
+// keys). A pass is bound by the ranking's instructions and the look-back's
+// latency. (Three
+// kernels per pass over 2048-key blocks -- counts, one scan per digit,
+// scatter -- took 83 us for the three passes of 1M keys and some 40 us for
+// 10k, where launches dominate.)
 // Item counts may live on the device (culled-in count, pair count), so grids
 // are sized for the capacity and blocks past the count exit early.
 #include "lf_internal.cuh"
@@ -36,29 +44,12 @@ namespace lf {
 
 namespace {
 
-constexpr int kThreads = 256;
-constexpr int kWarps = kThreads / 32;
 constexpr int kBits = 8;
-constexpr int kDigits = 1 << kBits;             // 256 = one digit per thread
-constexpr int kKPT = kRadixBlockKeys / kThreads; // 8 keys per thread
+constexpr int kDigits = 1 << kBits;
+constexpr int kWarps = kSweepThreads / 32;
 constexpr int kDepthKeyBits = 24;                // truncated depth key width
-constexpr int kDepthPasses = (kDepthKeyBits + kBits - 1) / kBits;
-static_assert(kDigits == kThreads, "one digit per thread in the digit scans");
-
-struct PassArgs {
-    long long n_static;                    // upper bound / fixed count
-    const unsigned long long* n_dev;       // device count (or null)
-    const unsigned long long* kmin;        // valid depth-key range (depth sort) or null
-    const unsigned long long* kmax;
-    int shift;
-    int first;                             // depth sort: drop the invalid key (all ones); value = index
-    int nb;                                // number of blocks (histogram stride)
-};
-
-__device__ __forceinline__ long long pass_count(const PassArgs& a)
-{
-    return a.n_dev ? (long long)*a.n_dev : a.n_static;
-}
+constexpr uint32_t kDepthKeyMask = (1u << kDepthKeyBits) - 1u;
+static_assert(kDepthPasses * kBits == kDepthKeyBits, "digits of the truncated depth key");
 
 // Right shift that keeps the top kDepthKeyBits varying bits of a depth key
 // relative to the smallest valid key (0 if the range already fits).
@@ -67,30 +58,6 @@ __device__ __forceinline__ int depth_shift(unsigned long long lo, unsigned long 
     if (lo > hi) return 0;
     const int bits = 64 - __clzll((long long)(hi - lo));
     return bits > kDepthKeyBits ? bits - kDepthKeyBits : 0;
-}
-
-// every valid truncated depth key has the same digit at this shift: identity pass
-__device__ __forceinline__ bool pass_uniform(const PassArgs& a)
-{
-    if (a.first || !a.kmin) return false;
-    const unsigned long long lo = *a.kmin, hi = *a.kmax;
-    if (lo > hi) return true;   // no valid keys
-    return (((hi - lo) >> depth_shift(lo, hi)) >> a.shift) == 0ull;
-}
-
-template <typename K>
-__device__ __forceinline__ uint32_t digit_of(K k, int shift)
-{
-    return (uint32_t)(k >> shift) & (uint32_t)(kDigits - 1);
-}
-
-// the key as sorted; false if absent (past the count, or culled)
-template <typename K>
-__device__ __forceinline__ bool load_key(const K* keys, long long idx, long long n, const PassArgs& a, K& k)
-{
-    if (idx >= n) return false;
-    k = keys[idx];
-    return !(a.first && k == (K)~(K)0);
 }
 
 // lanes holding the same digit (ballot per digit bit); valid lanes only
@@ -106,82 +73,8 @@ __device__ __forceinline__ uint32_t match_digit(uint32_t d, bool ok)
     return peers;
 }
 
-template <typename K>
-__global__ void __launch_bounds__(kThreads) k_upsweep(const K* __restrict__ keys, PassArgs a, uint32_t* hist)
-{
-    pdl_wait();
-    pdl_trigger();
-    __shared__ uint32_t h[kDigits];
-    if (pass_uniform(a)) return;
-    const long long n = pass_count(a);
-    if ((long long)blockIdx.x * kRadixBlockKeys >= n) {   // past the device count: empty histogram
-        hist[(size_t)threadIdx.x * a.nb + blockIdx.x] = 0u;
-        return;
-    }
-    h[threadIdx.x] = 0;
-    __syncthreads();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const long long base = (long long)blockIdx.x * kRadixBlockKeys + warp * (32 * kKPT);
-    K kk[kKPT];
-    uint32_t okm = 0;
-#pragma unroll
-    for (int r = 0; r < kKPT; ++r) {
-        K k = 0;
-        okm |= load_key(keys, base + r * 32 + lane, n, a, k) ? (1u << r) : 0u;
-        kk[r] = k;
-    }
-#pragma unroll
-    for (int r = 0; r < kKPT; ++r) {
-        const bool ok = (okm >> r) & 1u;
-        const uint32_t d = ok ? digit_of(kk[r], a.shift) : 0u;
-        const uint32_t peers = match_digit(d, ok);
-        if (ok && (__ffs(peers) - 1) == lane) atomicAdd(&h[d], (uint32_t)__popc(peers));
-    }
-    __syncthreads();
-    hist[(size_t)threadIdx.x * a.nb + blockIdx.x] = h[threadIdx.x];
-}
-
-// Exclusive scan of digit row d (hist[d * nb + b] over blocks b), in place;
-// the row total goes to tot[d].
-__global__ void __launch_bounds__(kThreads) k_rowscan(uint32_t* hist, uint32_t* tot, PassArgs a)
-{
-    pdl_wait();
-    pdl_trigger();
-    if (pass_uniform(a)) return;
-    __shared__ uint32_t warp_tot[kWarps];
-    uint32_t* row = hist + (size_t)blockIdx.x * a.nb;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    // blocks past the device count hold no keys (their downsweep exits)
-    const long long n = pass_count(a);
-    const int nb = (int)min((long long)a.nb, (n + kRadixBlockKeys - 1) / kRadixBlockKeys);
-    uint32_t carry = 0;
-    for (int base = 0; base < nb; base += kThreads) {
-        const int i = base + threadIdx.x;
-        const uint32_t v = i < nb ? row[i] : 0u;
-        uint32_t x = v;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t u = __shfl_up_sync(0xffffffffu, x, o);
-            if (lane >= o) x += u;
-        }
-        if (lane == 31) warp_tot[warp] = x;
-        __syncthreads();
-        uint32_t before = 0, total = 0;
-#pragma unroll
-        for (int w = 0; w < kWarps; ++w) {
-            const uint32_t t = warp_tot[w];
-            before += w < warp ? t : 0u;
-            total += t;
-        }
-        if (i < nb) row[i] = carry + before + x - v;
-        carry += total;
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) tot[blockIdx.x] = carry;
-}
-
-// exclusive scan of one value per thread over the block; returns the total
-__device__ __forceinline__ uint32_t block_exscan(uint32_t v, uint32_t* warp_tmp, uint32_t* total)
+// exclusive scan of one value per thread over the block; every thread calls it
+__device__ __forceinline__ uint32_t block_exscan(uint32_t v, uint32_t* warp_tmp)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint32_t x = v;
@@ -193,85 +86,117 @@ __device__ __forceinline__ uint32_t block_exscan(uint32_t v, uint32_t* warp_tmp,
     __syncthreads();
     if (lane == 31) warp_tmp[warp] = x;
     __syncthreads();
-    uint32_t before = 0, tot = 0;
+    uint32_t before = 0;
 #pragma unroll
-    for (int w = 0; w < kWarps; ++w) {
-        const uint32_t t = warp_tmp[w];
-        before += w < warp ? t : 0u;
-        tot += t;
-    }
-    *total = tot;
+    for (int w = 0; w < kWarps; ++w) before += w < warp ? warp_tmp[w] : 0u;
     return before + x - v;
 }
 
-template <typename K>
-struct DownSmem {
-    uint32_t wcnt[kWarps][kDigits];       // per-warp digit counts, then per-warp offsets
-    uint32_t blk_start[kDigits];          // block-local start of every digit run
-    uint32_t glob_base[kDigits];          // global destination of every digit run
-    K xkey[kRadixBlockKeys];              // exchange buffer in block-local digit order
-    uint32_t xval[kRadixBlockKeys];
-    uint32_t warp_tmp[kWarps];
-};
-
-template <typename K>
-__global__ void __launch_bounds__(kThreads) k_downsweep(const K* __restrict__ kin, const uint32_t* __restrict__ vin,
-                                                        K* __restrict__ kout, uint32_t* __restrict__ vout,
-                                                        PassArgs a, const uint32_t* __restrict__ hist,
-                                                        const uint32_t* __restrict__ tot)
+// Digit totals of the three depth passes over the culled-in keys.
+constexpr int kHistKeys = 16;   // keys per thread
+__global__ void __launch_bounds__(kSweepThreads) k_depth_hist(BuildWs w, long long n)
 {
     pdl_wait();
     pdl_trigger();
-    extern __shared__ __align__(16) unsigned char dsm_raw[];
-    DownSmem<K>& S = *reinterpret_cast<DownSmem<K>*>(dsm_raw);
-    const long long n = pass_count(a);
-    const long long blk = (long long)blockIdx.x * kRadixBlockKeys;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (pass_uniform(a)) {
-        // every key has the same digit: the stable permutation is the identity
-        for (int i = threadIdx.x; i < kRadixBlockKeys; i += kThreads) {
-            const long long idx = blk + i;
-            if (idx < n) {
-                kout[idx] = kin[idx];
-                vout[idx] = vin[idx];
-            }
-        }
-        return;
-    }
-    if (blk >= n) return;
-    const int d0 = threadIdx.x;   // the digit this thread scans
-
+    __shared__ uint32_t h[kDepthPasses][kDigits];
+    for (int i = threadIdx.x; i < kDepthPasses * kDigits; i += kSweepThreads) (&h[0][0])[i] = 0u;
+    const unsigned long long lo = w.hdr->kmin;
+    const int shift = depth_shift(lo, w.hdr->kmax);
+    __syncthreads();
+    const long long base = (long long)blockIdx.x * (kSweepThreads * kHistKeys);
+    unsigned long long k[kHistKeys];
 #pragma unroll
-    for (int w = 0; w < kWarps; ++w) S.wcnt[w][d0] = 0;
-    {
-        uint32_t total;
-        S.glob_base[d0] = block_exscan(tot[d0], S.warp_tmp, &total) + hist[(size_t)d0 * a.nb + blockIdx.x];
+    for (int r = 0; r < kHistKeys; ++r) {
+        const long long i = base + r * kSweepThreads + threadIdx.x;
+        k[r] = i < n ? w.keyA[i] : kInvalidKey;
+    }
+#pragma unroll
+    for (int r = 0; r < kHistKeys; ++r) {
+        if (k[r] == kInvalidKey) continue;
+        const uint32_t t = (uint32_t)((k[r] - lo) >> shift);
+#pragma unroll
+        for (int q = 0; q < kDepthPasses; ++q) atomicAdd(&h[q][(t >> (q * kBits)) & (kDigits - 1)], 1u);
     }
     __syncthreads();
+    for (int i = threadIdx.x; i < kDepthPasses * kDigits; i += kSweepThreads) {
+        const uint32_t c = (&h[0][0])[i];
+        if (c) atomicAdd(&w.dhist[i], c);
+    }
+}
 
-    // rank: warp w owns keys [512 w, 512 w + 512) of the block, visited in
+struct SweepArgs {
+    WsHeader* hdr;
+    long long n_static;                    // number of keys, unless n_dev
+    const unsigned long long* n_dev;       // device count (or null)
+    int shift;
+    int pass;                              // ticket
+    const uint32_t* tot;                   // digit totals of this pass
+    unsigned long long* stat;              // look-back words [blocks][kDigits]
+};
+
+constexpr int kLook = 16;   // predecessors per round trip of the look-back
+
+template <int KPT>
+struct SweepSmem {
+    uint32_t wcnt[kWarps][kDigits];       // per-warp digit counts, then per-warp offsets
+    uint32_t blk_start[kDigits];          // block-local start of every digit run
+    uint32_t glob_base[kDigits];          // global destination of every digit run
+    uint32_t xkey[kSweepThreads * KPT];   // exchange buffer in block-local digit order
+    uint32_t xval[kSweepThreads * KPT];
+    uint32_t warp_tmp[kWarps];
+    uint32_t tile, placed;
+};
+
+// One pass. FIRST (depth): the keys are the truncated forms of the 64-bit
+// keys at kin, culled ones dropped; a key's value is its index.
+template <int KPT, bool FIRST>
+__global__ void __launch_bounds__(kSweepThreads, 2) k_sweep(const void* __restrict__ kin, const uint32_t* __restrict__ vin,
+                                                         uint32_t* __restrict__ kout, uint32_t* __restrict__ vout,
+                                                         SweepArgs a)
+{
+    pdl_wait();
+    pdl_trigger();
+    extern __shared__ __align__(16) unsigned char sweep_raw[];
+    SweepSmem<KPT>& S = *reinterpret_cast<SweepSmem<KPT>*>(sweep_raw);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const long long n = a.n_dev ? (long long)*a.n_dev : a.n_static;
+    if (tid == 0) S.tile = atomicAdd(&a.hdr->ticket[a.pass], 1u);
+    for (int i = tid; i < kWarps * kDigits; i += kSweepThreads) (&S.wcnt[0][0])[i] = 0u;
+    __syncthreads();
+    const long long tile = S.tile, blk = tile * (kSweepThreads * KPT);
+    if (blk >= n) return;
+
+    // warp w owns keys [32 KPT w, 32 KPT (w + 1)) of the block, visited in
     // order round by round, so equal digits keep their order
-    K key[kKPT];
-    uint32_t val[kKPT], dig[kKPT], pos[kKPT];
-    const long long wbase = blk + warp * (32 * kKPT);
-    const uint32_t lt = (1u << lane) - 1u;
-    // all loads first (the ranking rounds below synchronise the warp)
+    uint32_t key[KPT], val[KPT], pos[KPT];
     uint32_t okm = 0;
-#pragma unroll
-    for (int r = 0; r < kKPT; ++r) {
-        const long long idx = wbase + r * 32 + lane;
-        K k = 0;
-        const bool ok = load_key(kin, idx, n, a, k);
-        key[r] = k;
-        val[r] = ok ? (a.first ? (uint32_t)idx : vin[idx]) : 0u;
-        okm |= ok ? (1u << r) : 0u;
+    const long long wbase = blk + warp * (32 * KPT);
+    unsigned long long lo = 0;
+    int dshift = 0;
+    if (FIRST) {
+        lo = a.hdr->kmin;
+        dshift = depth_shift(lo, a.hdr->kmax);
     }
 #pragma unroll
-    for (int r = 0; r < kKPT; ++r) {
+    for (int r = 0; r < KPT; ++r) {
+        const long long idx = wbase + r * 32 + lane;
+        bool ok = idx < n;
+        if (FIRST) {
+            const unsigned long long k = ok ? static_cast<const unsigned long long*>(kin)[idx] : kInvalidKey;
+            ok = k != kInvalidKey;
+            key[r] = (uint32_t)((k - lo) >> dshift);
+            val[r] = (uint32_t)idx;
+        } else {
+            key[r] = ok ? static_cast<const uint32_t*>(kin)[idx] : 0u;
+            val[r] = ok ? vin[idx] : 0u;
+        }
+        okm |= ok ? (1u << r) : 0u;
+    }
+    const uint32_t lt = (1u << lane) - 1u;
+#pragma unroll
+    for (int r = 0; r < KPT; ++r) {
         const bool ok = (okm >> r) & 1u;
-        const K k = key[r];
-        const uint32_t d = ok ? digit_of(k, a.shift) : 0u;
-        dig[r] = ok ? d : (uint32_t)kDigits;
+        const uint32_t d = ok ? (key[r] >> a.shift) & (kDigits - 1u) : 0u;
         const uint32_t peers = match_digit(d, ok);
         const uint32_t before = ok ? S.wcnt[warp][d] : 0u;
         __syncwarp();
@@ -280,30 +205,62 @@ __global__ void __launch_bounds__(kThreads) k_downsweep(const K* __restrict__ ki
         __syncwarp();
     }
     __syncthreads();
-    // per digit: exclusive offsets over warps and the block-local digit total
+    // per digit: exclusive offsets over warps and the block's count, published at once
     uint32_t run = 0;
+    if (tid < kDigits) {
 #pragma unroll
-    for (int w = 0; w < kWarps; ++w) {
-        const uint32_t c = S.wcnt[w][d0];
-        S.wcnt[w][d0] = run;
-        run += c;
+        for (int w = 0; w < kWarps; ++w) {
+            const uint32_t c = S.wcnt[w][tid];
+            S.wcnt[w][tid] = run;
+            run += c;
+        }
+        st_word(a.stat + (size_t)tile * kDigits + tid, (tile == 0 ? kSumAll : kSumOwn) | run);
     }
-    uint32_t placed;
-    S.blk_start[d0] = block_exscan(run, S.warp_tmp, &placed);
-    __syncthreads();
+    const uint32_t start = block_exscan(tid < kDigits ? run : 0u, S.warp_tmp);
+    if (tid < kDigits) S.blk_start[tid] = start;
+    if (tid == kDigits - 1) S.placed = start + run;
+    const uint32_t dbase = block_exscan(tid < kDigits ? a.tot[tid] : 0u, S.warp_tmp);   // orders blk_start, too
     // exchange into block-local digit order
 #pragma unroll
-    for (int r = 0; r < kKPT; ++r) {
-        if (dig[r] >= (uint32_t)kDigits) continue;
-        const uint32_t l = S.blk_start[dig[r]] + S.wcnt[warp][dig[r]] + pos[r];
+    for (int r = 0; r < KPT; ++r) {
+        if (!((okm >> r) & 1u)) continue;
+        const uint32_t d = (key[r] >> a.shift) & (kDigits - 1u);
+        const uint32_t l = S.blk_start[d] + S.wcnt[warp][d] + pos[r];
         S.xkey[l] = key[r];
         S.xval[l] = val[r];
     }
+    if (tid < kDigits) {
+        unsigned long long sum = 0;
+        long long t = tile - 1;
+        int idle = 0;
+        bool done = tile == 0;
+        while (!done) {
+            unsigned long long v[kLook];
+#pragma unroll
+            for (int u = 0; u < kLook; ++u)
+                v[u] = t - u >= 0 ? ld_word(a.stat + (size_t)(t - u) * kDigits + tid) : kSumAll;
+            int u = 0;
+#pragma unroll
+            for (int e = 0; e < kLook; ++e) {
+                if (u != e || done || v[e] < kSumOwn) continue;   // in order, up to the first word not there yet
+                sum += v[e] & kSumMask;
+                done = v[e] >= kSumAll;
+                ++u;
+            }
+            t -= u;
+            idle = u ? 0 : idle + 1;
+            if (idle > kLookbackTries) {
+                atomicExch(&a.hdr->timeout, 1);
+                done = true;
+            }
+        }
+        if (tile > 0) st_word(a.stat + (size_t)tile * kDigits + tid, kSumAll | (sum + run));
+        S.glob_base[tid] = dbase + (uint32_t)sum;
+    }
     __syncthreads();
     // coalesced write-out: item l of digit d goes to glob_base[d] + (l - blk_start[d])
-    for (uint32_t l = threadIdx.x; l < placed; l += kThreads) {
-        const K k = S.xkey[l];
-        const uint32_t d = digit_of(k, a.shift);
+    for (uint32_t l = tid; l < S.placed; l += kSweepThreads) {
+        const uint32_t k = S.xkey[l], d = (k >> a.shift) & (kDigits - 1u);
         const uint32_t dst = S.glob_base[d] + (l - S.blk_start[d]);
         kout[dst] = k;
         vout[dst] = S.xval[l];
@@ -312,20 +269,6 @@ __global__ void __launch_bounds__(kThreads) k_downsweep(const K* __restrict__ ki
 
 // ---- depth order ---------------------------------------------------------
 
-// truncated 32-bit depth key of every primitive (all ones if culled)
-__global__ void __launch_bounds__(256) k_depth_key32(const unsigned long long* __restrict__ key64,
-                                                     uint32_t* __restrict__ k32, long long n,
-                                                     const WsHeader* __restrict__ hdr)
-{
-    pdl_wait();
-    pdl_trigger();
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const unsigned long long lo = hdr->kmin, hi = hdr->kmax;
-    const unsigned long long k = key64[i];
-    k32[i] = k == kInvalidKey ? 0xffffffffu : (uint32_t)((k - lo) >> depth_shift(lo, hi));
-}
-
 // (full key, index) order of two ranks' primitives
 __device__ __forceinline__ bool depth_less(unsigned long long ka, uint32_t va, unsigned long long kb, uint32_t vb)
 {
@@ -333,72 +276,58 @@ __device__ __forceinline__ bool depth_less(unsigned long long ka, uint32_t va, u
 }
 
 constexpr int kShortRun = 32;
-constexpr int kLongRunCtas = 304;
+constexpr int kLongRunCtas = 152;
 constexpr int kLongRunThreads = 1024;
 constexpr int kSmemRun = 2048;
 
-// Within a run of equal truncated keys the ranks are in index order (the
-// sort is stable), so the run is already in (full key, index) order unless
-// some neighbour pair has a larger full key first. One flag per rank marks
-// such pairs (bytes over keyB, free at this point).
-__global__ void __launch_bounds__(256) k_depth_bad(BuildWs w)
+// The sorted ranks (tkeyB, valB) into (full key, index) order (valA). A rank
+// alone with its truncated key is copied. The members of a run of up to
+// kShortRun equal truncated keys each count the members before them. Longer
+// runs are copied (the sort is stable: they are in index order, which is right
+// unless some neighbour pair has a larger full key first); a member that finds
+// such a pair claims its run (top bit of the run's first key) and the first
+// claim lists it in tkeyA for k_depth_long_runs. (Out of place: no rank reads
+// what another one writes.)
+__global__ void __launch_bounds__(256) k_depth_runs(BuildWs w)
 {
     pdl_wait();
     pdl_trigger();
     const long long M = (long long)w.hdr->M;
     const long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= M) return;
-    uint8_t b = 0;
-    if (r > 0 && w.tkeyA[r] == w.tkeyA[r - 1]) b = w.keyA[w.valA[r - 1]] > w.keyA[w.valA[r]] ? 1 : 0;
-    reinterpret_cast<uint8_t*>(w.keyB)[r] = b;
-}
-
-// Runs of equal truncated keys that hold an out-of-order pair. Work starts
-// at flagged ranks only: a flagged rank walks back to its run's start and
-// leaves if it meets an earlier flag (that one owns the run), so every run
-// is owned once and walked once. The owner finds the run's end, sorts a run
-// of up to kShortRun keys itself and lists longer ones (start, length) in
-// tkeyB. Runs with no flag (equal keys, e.g. primitives on one grid layer)
-// cost nothing.
-__global__ void __launch_bounds__(256) k_depth_runs(BuildWs w)
-{
-    pdl_wait();
-    pdl_trigger();
-    const long long M = (long long)w.hdr->M;
-    const long long r0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const uint8_t* bad = reinterpret_cast<const uint8_t*>(w.keyB);
-    if (r0 >= M || !bad[r0]) return;
-    const uint32_t* k = w.tkeyA;
-    const uint32_t kr = k[r0];
-    long long r = r0 - 1;                         // candidate run start
-    while (r > 0 && k[r - 1] == kr) {
-        if (bad[r]) return;                       // an earlier flag owns this run
-        --r;
-    }
-    long long e = r0 + 1;
-    while (e < M && k[e] == kr) ++e;
-    const int L = (int)min(e - r, (long long)0x7fffffff);
-    if (L > kShortRun) {
-        const unsigned long long q = atomicAdd(&w.hdr->long_runs, 1ull);
-        w.tkeyB[2 * q] = (uint32_t)r;
-        w.tkeyB[2 * q + 1] = (uint32_t)L;
+    const uint32_t* key = w.tkeyB;
+    auto same = [&](long long i, uint32_t k) { return i >= 0 && i < M && ((key[i] ^ k) & kDepthKeyMask) == 0u; };
+    const uint32_t k = key[r], v = min(w.valB[r], (uint32_t)(w.hdr->n - 1));   // (in bounds after a wait gave up, too)
+    const bool left = same(r - 1, k), right = same(r + 1, k);
+    if (!left && !right) {
+        w.valA[r] = v;
         return;
     }
-    unsigned long long kk[kShortRun];
-    uint32_t vv[kShortRun];
-    for (int i = 0; i < L; ++i) {
-        const uint32_t v = w.valA[r + i];
-        const unsigned long long key = w.keyA[v];
-        int j = i;
-        while (j > 0 && depth_less(key, v, kk[j - 1], vv[j - 1])) {
-            kk[j] = kk[j - 1];
-            vv[j] = vv[j - 1];
-            --j;
-        }
-        kk[j] = key;
-        vv[j] = v;
+    long long s = r, e = r + 1;   // the run, as far as kShortRun from here
+    bool longer = same(r - kShortRun, k) || same(r + kShortRun, k);
+    if (!longer) {
+        while (same(s - 1, k)) --s;
+        while (same(e, k)) ++e;
+        longer = e - s > kShortRun;
     }
-    for (int i = 0; i < L; ++i) w.valA[r + i] = vv[i];
+    const unsigned long long full = w.keyA[v];
+    if (!longer) {
+        int before = 0;
+        for (long long i = s; i < e; ++i) {
+            const uint32_t u = min(w.valB[i], (uint32_t)(w.hdr->n - 1));
+            before += i != r && depth_less(w.keyA[u], u, full, v) ? 1 : 0;
+        }
+        w.valA[s + before] = v;
+        return;
+    }
+    w.valA[r] = v;
+    if (!left || w.keyA[min(w.valB[r - 1], (uint32_t)(w.hdr->n - 1))] <= full) return;
+    for (s = r; same(s - 1, k);) --s;
+    if (atomicOr(&w.tkeyB[s], 0x80000000u) & 0x80000000u) return;   // listed
+    while (same(e, k)) ++e;
+    const unsigned long long q = atomicAdd(&w.hdr->long_runs, 1ull);
+    w.tkeyA[2 * q] = (uint32_t)s;
+    w.tkeyA[2 * q + 1] = (uint32_t)(e - s);
 }
 
 // Batcher's odd-even merge network over P = 2^m slots: every comparator puts
@@ -421,8 +350,8 @@ __global__ void __launch_bounds__(kLongRunThreads) k_depth_long_runs(BuildWs w)
     __shared__ uint32_t sv[kSmemRun];
     const unsigned long long nr = w.hdr->long_runs;
     for (unsigned long long q = blockIdx.x; q < nr; q += gridDim.x) {
-        const long long r = w.tkeyB[2 * q];
-        const long long L = w.tkeyB[2 * q + 1];
+        const long long r = w.tkeyA[2 * q];
+        const long long L = w.tkeyA[2 * q + 1];
         long long P = 1;
         while (P < L) P <<= 1;
         if (P <= kSmemRun) {
@@ -471,45 +400,59 @@ __global__ void __launch_bounds__(kLongRunThreads) k_depth_long_runs(BuildWs w)
     }
 }
 
-template <typename K>
-void radix_pass(const K* kin, const uint32_t* vin, K* kout, uint32_t* vout, const PassArgs& a, uint32_t* hist,
-                uint32_t* tot, cudaStream_t s)
+template <int KPT, bool FIRST>
+void sweep_kpt_launch(const void* kin, const uint32_t* vin, uint32_t* kout, uint32_t* vout, const SweepArgs& a,
+                      long long blocks, cudaStream_t s)
 {
-    cudaFuncSetAttribute(k_downsweep<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(DownSmem<K>));
-    launch_pdl(k_upsweep<K>, dim3(a.nb), dim3(kThreads), 0, s, kin, a, hist);
-    launch_pdl(k_rowscan, dim3(kDigits), dim3(kThreads), 0, s, hist, tot, a);
-    launch_pdl(k_downsweep<K>, dim3(a.nb), dim3(kThreads), sizeof(DownSmem<K>), s, kin, vin, kout, vout, a, hist, tot);
-    note_launches(3);
+    cudaFuncSetAttribute(k_sweep<KPT, FIRST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SweepSmem<KPT>));
+    launch_pdl(k_sweep<KPT, FIRST>, dim3((unsigned)blocks), dim3(kSweepThreads), sizeof(SweepSmem<KPT>), s, kin, vin, kout,
+               vout, a);
+    note_launches(1);
+}
+
+template <bool FIRST>
+void sweep(int kpt, const void* kin, const uint32_t* vin, uint32_t* kout, uint32_t* vout, const SweepArgs& a,
+           long long blocks, cudaStream_t s)
+{
+    if (kpt == 4)
+        sweep_kpt_launch<4, FIRST>(kin, vin, kout, vout, a, blocks, s);
+    else
+        sweep_kpt_launch<8, FIRST>(kin, vin, kout, vout, a, blocks, s);
 }
 
 }  // namespace
 
+int sweep_kpt(long long n)
+{
+    return n <= 152ll * kSweepThreads * 4 ? 4 : 8;
+}
+
 void sort_depth_keys(const BuildWs& ws, long long n, cudaStream_t s)
 {
     if (n <= 0) return;
-    const int nb = (int)((n + kRadixBlockKeys - 1) / kRadixBlockKeys);
-    uint32_t* kb[2] = {ws.tkeyA, ws.tkeyB};
-    uint32_t* vb[2] = {ws.valA, ws.valB};
-    // start in the buffer that makes the last pass end in tkeyA / valA
-    int cur = kDepthPasses & 1;
-    launch_pdl(k_depth_key32, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, s, ws.keyA, kb[cur], n, ws.hdr);
+    const long long per = kSweepThreads * kHistKeys;
+    launch_pdl(k_depth_hist, dim3((unsigned)((n + per - 1) / per)), dim3(kSweepThreads), 0, s, ws, n);
+    // the passes end in tkeyB / valB
+    uint32_t* kb[2] = {ws.tkeyB, ws.tkeyA};
+    uint32_t* vb[2] = {ws.valB, ws.valA};
     for (int pass = 0; pass < kDepthPasses; ++pass) {
-        PassArgs a;
+        SweepArgs a;
+        a.hdr = ws.hdr;
         a.n_static = n;
         a.n_dev = pass == 0 ? nullptr : &ws.hdr->M;
-        a.kmin = &ws.hdr->kmin;
-        a.kmax = &ws.hdr->kmax;
         a.shift = pass * kBits;
-        a.first = pass == 0;
-        a.nb = nb;
-        radix_pass<uint32_t>(kb[cur], vb[cur], kb[cur ^ 1], vb[cur ^ 1], a, ws.hist, ws.dtot, s);
-        cur ^= 1;
+        a.pass = pass;
+        a.tot = ws.dhist + pass * kDigits;
+        a.stat = ws.sstat + (size_t)pass * ws.nb_depth * kDigits;
+        const int in = (pass + 1) & 1, out = pass & 1;
+        if (pass == 0)
+            sweep<true>(ws.kpt_depth, ws.keyA, nullptr, kb[out], vb[out], a, ws.nb_depth, s);
+        else
+            sweep<false>(ws.kpt_depth, kb[in], vb[in], kb[out], vb[out], a, ws.nb_depth, s);
     }
-    // truncated keys in tkeyA, ranks in valA; now the runs
-    launch_pdl(k_depth_bad, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, s, ws);
     launch_pdl(k_depth_runs, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, s, ws);
     launch_pdl(k_depth_long_runs, dim3(kLongRunCtas), dim3(kLongRunThreads), 0, s, ws);
-    note_launches(4);
+    note_launches(3);
 }
 
 int tile_sort_passes(int tile_bits) { return (tile_bits + kBits - 1) / kBits; }
@@ -520,20 +463,17 @@ void sort_tile_keys(const BuildWs& ws, long long cap, int tile_bits, cudaStream_
     uint32_t* kb[2] = {ws.tkeyA, ws.tkeyB};
     uint32_t* vb[2] = {ws.entA, ws.entB};
     int cur = 0;
-    if (cap > 0) {
-        const int nb = (int)((cap + kRadixBlockKeys - 1) / kRadixBlockKeys);
-        for (int pass = 0; pass < tile_sort_passes(tile_bits); ++pass) {
-            PassArgs a;
-            a.n_static = cap;
-            a.n_dev = &ws.hdr->tile_n;
-            a.kmin = nullptr;
-            a.kmax = nullptr;
-            a.shift = pass * kBits;
-            a.first = 0;
-            a.nb = nb;
-            radix_pass<uint32_t>(kb[cur], vb[cur], kb[cur ^ 1], vb[cur ^ 1], a, ws.hist, ws.dtot, s);
-            cur ^= 1;
-        }
+    for (int pass = 0; cap > 0 && pass < tile_sort_passes(tile_bits); ++pass) {
+        SweepArgs a;
+        a.hdr = ws.hdr;
+        a.n_static = cap;
+        a.n_dev = &ws.hdr->tile_n;
+        a.shift = pass * kBits;
+        a.pass = kDepthPasses + pass;
+        a.tot = ws.dhist + (kDepthPasses + pass) * kDigits;
+        a.stat = ws.sstat + ((size_t)kDepthPasses * ws.nb_depth + (size_t)pass * ws.nb_tile) * kDigits;
+        sweep<false>(ws.kpt_tile, kb[cur], vb[cur], kb[cur ^ 1], vb[cur ^ 1], a, ws.nb_tile, s);
+        cur ^= 1;
     }
     *keys_out = kb[cur];
     *vals_out = vb[cur];
