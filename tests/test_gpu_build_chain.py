@@ -107,3 +107,20 @@ def test_disparity_bins_at_their_edges(orc):
     sc.means[:, :2] *= (z / sc.means[:, 2])[:, None]
     sc.means[:, 2] = np.clip(z, zn, zf)
     _check(orc, sc, orc.gauss_decide, (256, 256), N, "disparity")
+
+
+@pytest.mark.parametrize("base,origin", [(1.0, (-0.4, -0.4, 1.5)), (0.3, (0.0, 0.0, 2.0)), (2.0 ** -1000, (0.1, 0.0, 2.0)),
+                                         (1e30, (0.0, 0.0, 3.0))])
+def test_voxel_projection_on_number_bits(orc, base, origin):
+    """Levels from 0 to 255, indices of every size and sign, sides down to the
+    subnormals: the projection's exponent and rounding steps give the FP64 and
+    FP32 results bit for bit."""
+    rng = np.random.default_rng(11)
+    n = 6000
+    level = rng.integers(0, 256, n) if base != 1.0 else rng.integers(0, 13, n)
+    lim = np.minimum(2.0 ** np.minimum(level, 30), 2.0 ** 31 - 1)
+    ijk = np.floor(rng.uniform(-1.0, 1.0, (n, 3)) * lim[:, None]).astype(np.int32)
+    ijk[:40] = 0
+    sc = S.VoxelScene(ijk, level.astype(np.uint8), np.asarray(origin, np.float64), float(base), np.ones((n, 8), np.float32),
+                      np.full((n, 3), 0.5, np.float32))
+    _check(orc, sc, orc.voxel_decide, (200, 150), 4, "quantile")
