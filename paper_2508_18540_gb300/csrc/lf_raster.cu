@@ -22,6 +22,8 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include <type_traits>
+
 #include "lf_internal.cuh"
 
 namespace lf {
@@ -86,27 +88,33 @@ __device__ __forceinline__ float ex2_approx(float x)
 // Gaussians. A CTA rasterises one (32 x 32 super-tile, chunk) list, or one
 // part of a long one, with 8 warps. Warp w owns the 8-column x 16-row strip
 // at column group w % 4 and row group w / 4 of the super-tile; lane l shades
-// column l % 8 in rows l / 8 + 4 s, s = 0 .. 3, so the lanes' s-th pixels
-// form the 8 x 4 sub-block s of the strip, and a footprint that misses a
-// sub-block costs the warp nothing there (sub-blocks of 32 pixels fit the
-// footprint sizes better than wide strips). Each batch of list entries is
-// staged as three 16-byte words {mean x, mean y, A, B}, {C, log2 o, cm, rm},
-// {r, g, b, wm}, with the conic pre-scaled so that
+// column l % 8 in rows l / 8 + 4 s, s = 0 .. 3. Slots 0, 1 and slots 2, 3 form
+// the strip's two 8 x 8 blocks, and each is one packed pair of FP32 lanes: the
+// kernel is bound by instruction issue, and the two-wide FMA, multiply and add
+// shade both pixels of a pair at once, with the rounding of the scalar ones.
+// Each batch of list entries is staged as {mean x, A, B, log2 o}, {-mean y
+// twice, C twice}, {r twice, g twice}, {b twice, cm, rm} and wm, with the conic
+// pre-scaled so that
 //   alpha = min(0.99, 2^(A dx^2 + B dx dy + C dy^2 + log2 o)),
 // A = -log2(e)/2 a, B = -log2(e) b, C = -log2(e)/2 c, and the footprint
 // rectangle as bit masks over the super-tile: bit c of cm for column c, bit r
-// of rm for row r, bit w of wm for the warps whose strips it meets (computed
-// once per entry and CTA, so a warp's visit tests bits instead of bounds).
-// Per visited entry a lane forms g1 = B dx and g0 = A dx^2 + log2 o for its
-// column once; each of its rows inside the footprint then costs the Horner
-// form (C dy + g1) dy + g0, one ex2 and the blend. Every warp ballots which
-// entries touch its strip and visits only those, in list order, so each
-// pixel blends its members front to back. Two staging buffers alternate: one
-// CTA barrier per batch.
+// of rm for row r, bits w and 8 + w of wm for the upper and lower block of warp
+// w's strip. A warp ballots the bits of 32 entries and visits only the blocks
+// that an entry meets, in list order; the ballots are uniform, so the visits
+// branch without divergence. Per visit a lane forms g1 = B dx and g0 = A dx^2
+// + log2 o for its column once; each block then costs the Horner form
+// (C dy + g1) dy + g0 and the blend of two pixels and two ex2. A pixel outside
+// the footprint blends with alpha 0, which leaves (C, T) as they are; entries
+// whose colour is not finite (0 inf = NaN) take a loop that selects. (One
+// divergent branch and scalar arithmetic per 8 x 4 sub-block took 65
+// instructions a visit.) Two staging buffers alternate: one CTA barrier per
+// batch.
 //
 // Load balance. The work of a list grows with its length, and dense regions
 // of the scene make a few lists far longer than the rest. k_raster_plan cuts
-// every list longer than r_seg entries into parts of r_seg entries, and
+// every list longer than r_seg entries into parts of r_seg entries (1024; in
+// frames of few pairs, where the longest list is the kernel's time, down to
+// one staged batch: the 10k-Gaussian frame 85 -> 82 us), and
 // k_raster_gauss_parts rasterises the parts: each blends its entries into a
 // partial (C, T) started from (0, 1) and stores it in its slot, and the CTA
 // that finishes a list's last part composes the partials in part order,
@@ -122,9 +130,63 @@ constexpr int kGaussThreads = 32 * 4 * (8 / kGaussNS);
 
 struct GaussSmem {
     float4 e0[2][kGaussThreads];
-    float4 e1[2][kGaussThreads];
-    float4 rgb[2][kGaussThreads];
+    ulonglong2 e1[2][kGaussThreads];
+    ulonglong2 e2[2][kGaussThreads];
+    float4 e3[2][kGaussThreads];
+    uint32_t wm[2][kGaussThreads];   // blocks met; bit 31: the colour is not finite
 };
+
+// two FP32 numbers in one 64-bit register pair, and their two-wide arithmetic
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 pack2(float a, float b)
+{
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(f32x2 v)
+{
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c)
+{
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b)
+{
+    f32x2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b)
+{
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
+// Columns cm and rows rm of the super-tile that footprint r covers, as bit masks.
+__device__ __forceinline__ void footprint_masks(int4 r, int SX, int SY, uint32_t* cm, uint32_t* rm)
+{
+    const int cl = max(r.x - SX, 0), ch = min(r.z - SX, kSuper - 1);
+    const int rl = max(r.y - SY, 0), rh = min(r.w - SY, kSuper - 1);
+    *cm = cl <= ch ? (0xffffffffu >> (31 - ch)) & (0xffffffffu << cl) : 0u;
+    *rm = rl <= rh ? (0xffffffffu >> (31 - rh)) & (0xffffffffu << rl) : 0u;
+}
+
+// bits w and 8 + w: the footprint meets the upper / lower 8 x 8 block of warp w's strip
+__device__ __forceinline__ uint32_t strip_blocks(uint32_t cm, uint32_t rm)
+{
+    uint32_t c4 = 0u;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) c4 |= (cm >> (8 * q)) & 0xffu ? 1u << q : 0u;
+    return ((rm & 0x000000ffu) ? c4 : 0u) | ((rm & 0x00ff0000u) ? c4 << 4 : 0u) |
+           ((rm & 0x0000ff00u) ? c4 << 8 : 0u) | ((rm & 0xff000000u) ? c4 << 12 : 0u);
+}
 
 // Split parts of one raster (one thread per (super-tile, chunk) list): a list
 // of L > r_seg entries takes P = ceil(L / r_seg) consecutive partial slots;
@@ -137,8 +199,8 @@ __global__ void __launch_bounds__(kPlanThreads) k_raster_plan(BuildWs w, int lis
     int S = 0x7fffffff;
     if (split) {
         long long need = (2 * total + w.r_nslots - 1) / w.r_nslots;   // keeps the parts within the slots
-        need = (need + 255) / 256 * 256;
-        S = (int)(need > kRasterSegMin ? need : kRasterSegMin);
+        need = max(need, min(total / kRasterCtas, (long long)kRasterSegMax));
+        S = (int)((max(need, (long long)kRasterSegMin) + 255) / 256 * 256);
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) w.hdr->r_seg = S;
     for (int id = blockIdx.x * kPlanThreads + threadIdx.x; id < lists; id += gridDim.x * kPlanThreads) {
@@ -178,10 +240,14 @@ __device__ __forceinline__ void raster_gauss_list(const BuildWs& w, const Raster
     const float fpx = (float)px;
     // bit of this lane's column in cm, of its slot-0 row in rm
     const int csh = px - SX, rsh = py0 - SY;
-    float C[NS][3], T[NS];
+    f32x2 Cn[2][3], T2[2], py2[2];   // -C, T and pixel rows of the pairs (slots 2 q, 2 q + 1)
     uint32_t stopped = 0u;
 #pragma unroll
-    for (int s = 0; s < NS; ++s) C[s][0] = C[s][1] = C[s][2] = 0.f, T[s] = 1.f;
+    for (int q = 0; q < 2; ++q) {
+        Cn[q][0] = Cn[q][1] = Cn[q][2] = 0ull;
+        T2[q] = pack2(1.f, 1.f);
+        py2[q] = pack2((float)(py0 + 8 * q), (float)(py0 + 8 * q + 4));
+    }
     int buf = 0;
     for (int base = 0; base < L; base += NT, buf ^= 1) {
         const int i = base + threadIdx.x;
@@ -190,67 +256,95 @@ __device__ __forceinline__ void raster_gauss_list(const BuildWs& w, const Raster
             const int4 r = w.r_rect[rk];
             const float4 geo = w.r_geo[rk];
             const float4 c = w.r_con[rk];
-            sm.e0[buf][threadIdx.x] = make_float4(geo.x, geo.y, -0.5f * kL2E * c.x, -kL2E * c.y);
-            // footprint columns / rows of the super-tile as bit masks, and
-            // the warps whose 8 x 16 strips it meets
-            const int cl = max(r.x - SX, 0), ch = min(r.z - SX, kSuper - 1);
-            const int rl = max(r.y - SY, 0), rh = min(r.w - SY, kSuper - 1);
-            const uint32_t cm = cl <= ch ? (0xffffffffu >> (31 - ch)) & (0xffffffffu << cl) : 0u;
-            const uint32_t rm = rl <= rh ? (0xffffffffu >> (31 - rh)) & (0xffffffffu << rl) : 0u;
-            uint32_t wm = 0u;
-#pragma unroll
-            for (int q = 0; q < 8; ++q)
-                wm |= ((cm >> (8 * (q & 3))) & 0xffu) && ((rm >> (16 * (q >> 2))) & 0xffffu) ? 1u << q : 0u;
-            sm.e1[buf][threadIdx.x] =
-                make_float4(-0.5f * kL2E * c.z, __log2f(c.w), __uint_as_float(cm), __uint_as_float(rm));
             const float4 rgb = w.r_rgb[rk];
-            sm.rgb[buf][threadIdx.x] = make_float4(rgb.x, rgb.y, rgb.z, __uint_as_float(wm));
+            uint32_t cm, rm;
+            footprint_masks(r, SX, SY, &cm, &rm);
+            const float cc = -0.5f * kL2E * c.z;
+            sm.e0[buf][threadIdx.x] = make_float4(geo.x, -0.5f * kL2E * c.x, -kL2E * c.y, __log2f(c.w));
+            sm.e1[buf][threadIdx.x] = make_ulonglong2(pack2(-geo.y, -geo.y), pack2(cc, cc));
+            sm.e2[buf][threadIdx.x] = make_ulonglong2(pack2(rgb.x, rgb.x), pack2(rgb.y, rgb.y));
+            sm.e3[buf][threadIdx.x] = make_float4(rgb.z, rgb.z, __uint_as_float(cm), __uint_as_float(rm));
+            const bool finite = isfinite(rgb.x) && isfinite(rgb.y) && isfinite(rgb.z);
+            sm.wm[buf][threadIdx.x] = strip_blocks(cm, rm) | (finite ? 0u : 0x80000000u);
         }
         // orders this batch's staging before its walk, and every warp's walk
         // of the batch before last before this staging overwrote its buffer
         __syncthreads();
         const int cnt = min(NT, L - base);
         const float4* s_e0 = sm.e0[buf];
-        const float4* s_e1 = sm.e1[buf];
-        const float4* s_rgb = sm.rgb[buf];
+        const ulonglong2* s_e1 = sm.e1[buf];
+        const ulonglong2* s_e2 = sm.e2[buf];
+        const float4* s_e3 = sm.e3[buf];
         for (int m0 = 0; m0 < cnt; m0 += 32) {
-            const int jl = m0 + lane;
-            const bool hit = jl < cnt && ((__float_as_uint(s_rgb[jl].w) >> warp) & 1u);
-            uint32_t mask = __ballot_sync(0xffffffffu, hit);
-            while (mask) {
-                const int j = m0 + __ffs(mask) - 1;
-                mask &= mask - 1;
-                const float4 e0 = s_e0[j];
-                const float4 e1 = s_e1[j];
-                const float4 col = s_rgb[j];
-                // slot s of this lane lies in the footprint iff bit 4 s of m is set
-                const uint32_t m = (__float_as_uint(e1.z) >> csh) & 1u ? __float_as_uint(e1.w) >> rsh : 0u;
-                const float dx = fpx - e0.x;
-                const float g1 = e0.w * dx;
-                const float g0 = fmaf(e0.z * dx, dx, e1.y);
-#pragma unroll
-                for (int s = 0; s < NS; ++s) {
-                    if (m & (1u << (4 * s))) {
-                        const float dy = (float)(py0 + 4 * s) - e0.y;
-                        const float pw = fmaf(fmaf(e1.x, dy, g1), dy, g0);
-                        const float al = fminf(0.99f, ex2_approx(pw));
-                        const float tn = fmaf(-T[s], al, T[s]);
+            const uint32_t wm = m0 + lane < cnt ? sm.wm[buf][m0 + lane] : 0u;
+            const uint32_t upper = __ballot_sync(0xffffffffu, (wm >> warp) & 1u);
+            const uint32_t lower = __ballot_sync(0xffffffffu, (wm >> (8 + warp)) & 1u);
+            auto walk = [&](auto finite) {
+                uint32_t mask = upper | lower;
+                while (mask) {
+                    const uint32_t bit = mask & (0u - mask);
+                    const int j = m0 + __ffs(mask) - 1;
+                    mask ^= bit;
+                    const float4 e0 = s_e0[j];
+                    const ulonglong2 e1 = s_e1[j];
+                    const ulonglong2 e2 = s_e2[j];
+                    const float4 e3 = s_e3[j];
+                    // slot s of this lane lies in the footprint iff bit 4 s of m is set
+                    uint32_t m = (__float_as_uint(e3.z) >> csh) & 1u ? __float_as_uint(e3.w) >> rsh : 0u;
+                    if (G3) m &= ~stopped;
+                    const float dx = fpx - e0.x;
+                    const float g1s = e0.z * dx;
+                    const float g0s = fmaf(e0.y * dx, dx, e0.w);
+                    const f32x2 g1 = pack2(g1s, g1s), g0 = pack2(g0s, g0s), blue = pack2(e3.x, e3.y);
+                    auto blend = [&](int q) {
+                        const f32x2 dy = add2(py2[q], e1.x);
+                        const float2 pw = unpack2(fma2(fma2(e1.y, dy, g1), dy, g0));
+                        const bool in0 = m & (1u << (8 * q)), in1 = m & (16u << (8 * q));
+                        // -alpha
+                        float n0 = in0 ? fmaxf(-0.99f, -ex2_approx(pw.x)) : 0.f;
+                        float n1 = in1 ? fmaxf(-0.99f, -ex2_approx(pw.y)) : 0.f;
                         if (G3) {
-                            if ((stopped >> s) & 1u) continue;
-                            if (al < 1.0f / 255.0f) continue;
-                            if (tn < 1e-4f) {
-                                stopped |= 1u << s;
-                                continue;
-                            }
+                            if (n0 > -1.0f / 255.0f) n0 = 0.f;
+                            if (n1 > -1.0f / 255.0f) n1 = 0.f;
+                            const float2 t = unpack2(T2[q]);
+                            const bool end0 = fmaf(t.x, n0, t.x) < 1e-4f, end1 = fmaf(t.y, n1, t.y) < 1e-4f;
+                            if (end0) n0 = 0.f, stopped |= 1u << (8 * q);
+                            if (end1) n1 = 0.f, stopped |= 16u << (8 * q);
                         }
-                        const float ta = T[s] * al;
-                        C[s][0] = fmaf(ta, col.x, C[s][0]);
-                        C[s][1] = fmaf(ta, col.y, C[s][1]);
-                        C[s][2] = fmaf(ta, col.z, C[s][2]);
-                        T[s] = tn;
-                    }
+                        const f32x2 na = pack2(n0, n1);
+                        const f32x2 nta = mul2(T2[q], na);
+                        f32x2 r = e2.x, g = e2.y, b = blue;
+                        if (!finite) {
+                            const bool on0 = G3 ? n0 != 0.f : in0, on1 = G3 ? n1 != 0.f : in1;
+                            const float2 rr = unpack2(r), gg = unpack2(g), bb = unpack2(b);
+                            r = pack2(on0 ? rr.x : 0.f, on1 ? rr.y : 0.f);
+                            g = pack2(on0 ? gg.x : 0.f, on1 ? gg.y : 0.f);
+                            b = pack2(on0 ? bb.x : 0.f, on1 ? bb.y : 0.f);
+                        }
+                        Cn[q][0] = fma2(nta, r, Cn[q][0]);
+                        Cn[q][1] = fma2(nta, g, Cn[q][1]);
+                        Cn[q][2] = fma2(nta, b, Cn[q][2]);
+                        T2[q] = fma2(T2[q], na, T2[q]);
+                    };
+                    if (upper & bit) blend(0);
+                    if (lower & bit) blend(1);
                 }
-            }
+            };
+            if (__any_sync(0xffffffffu, wm >> 31))
+                walk(std::false_type{});
+            else
+                walk(std::true_type{});
+        }
+    }
+    float C[NS][3], T[NS];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        const float2 t = unpack2(T2[q]);
+        T[2 * q] = t.x, T[2 * q + 1] = t.y;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const float2 v = unpack2(Cn[q][c]);
+            C[2 * q][c] = 0.f - v.x, C[2 * q + 1][c] = 0.f - v.y;
         }
     }
     if (SPLIT) {
@@ -291,9 +385,10 @@ __device__ __forceinline__ void raster_gauss_list(const BuildWs& w, const Raster
 }
 
 // Lists no longer than r_seg entries: one CTA per (super-tile x, chunk y).
-// The FP32 form takes 48 registers: five CTAs (40 warps) per SM. (A
-// minimum-blocks bound of five, same register count, measured 8 % slower;
-// only the 3DGS form, 58 registers unbounded, gains from it.)
+// 56 registers, four CTAs (32 warps) per SM; the 3DGS form is bounded to five.
+// (A bound of five for both: the 1M-Gaussian frame 890 us instead of 840, the
+// 10k one 90 instead of 85.) Scalar rows and divergent sub-blocks before: 894
+// and 100 us, and 934 instead of 821 for 500k Gaussians on 128 planes of 1024^2.
 // Launched behind the parts kernel, it does not wait for it to start;
 // CTA (0, 0) waits for it to finish before exiting, so this grid completes
 // after every part's texels are written and work ordered after it sees them.
@@ -311,7 +406,7 @@ __global__ void __launch_bounds__(kGaussThreads, G3 ? 5 : 0) k_raster_gauss(Buil
 
 // The parts of the split lists: CTA b takes item b (CTAs past r_heavy exit).
 // Bounded to 64 registers (four CTAs per SM; 66 unbounded, three): parts
-// dominate at few chunks (N = 16: 0.436 -> 0.398 ms).
+// dominate at few chunks (N = 16: 0.436 -> 0.398 ms with the scalar rows).
 // It lets the list kernel launch at once: that kernel reads nothing the
 // parts write.
 template <int DT>
