@@ -136,39 +136,6 @@ struct GaussSmem {
     uint32_t wm[2][kGaussThreads];   // blocks met; bit 31: the colour is not finite
 };
 
-// two FP32 numbers in one 64-bit register pair, and their two-wide arithmetic
-using f32x2 = unsigned long long;
-__device__ __forceinline__ f32x2 pack2(float a, float b)
-{
-    f32x2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ float2 unpack2(f32x2 v)
-{
-    float2 r;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-    return r;
-}
-__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c)
-{
-    f32x2 r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b)
-{
-    f32x2 r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b)
-{
-    f32x2 r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-
 // Columns cm and rows rm of the super-tile that footprint r covers, as bit masks.
 __device__ __forceinline__ void footprint_masks(int4 r, int SX, int SY, uint32_t* cm, uint32_t* rm)
 {
