@@ -69,3 +69,19 @@ def test_colour_that_is_not_finite_stays_in_its_footprint(blend, bad):
     assert same[..., [0, 2, 3]].all()                # the other channels everywhere
     changed = ~same[..., 1]
     assert changed.any() and not np.isfinite(b[..., 1][changed]).any()
+
+
+@pytest.mark.parametrize("corner", [(-0.4, -0.4), (0.1, -0.4), (0.1, 0.1)])
+def test_voxel_batches_without_hits(orc, corner):
+    """All voxels of a super-tile lie in one of its four tiles: the other
+    tiles go through several staged batches of its list without a hit."""
+    rng = np.random.default_rng(3)
+    n, cell = 1400, 0.04
+    cam, disp, views = _setup((32, 32))
+    ijk = np.floor(rng.uniform(0.0, 0.3, (n, 3)) / cell).astype(np.int32)
+    sc = S.VoxelScene(ijk, np.zeros(n, np.uint8), np.array([2 * corner[0], 2 * corner[1], 2.0]), cell,
+                      rng.uniform(0.0, 0.3, (n, 8)).astype(np.float32), rng.uniform(0.0, 1.0, (n, 3)).astype(np.float32))
+    o = orc.render(scene=sc, camera=cam, display=disp, views=views, N=1, binning="quantile")
+    gpu = G.run_gpu(sc, cam, disp, views, 1, "quantile")
+    assert gpu["status"] == 0 and np.array_equal(gpu["rect"], o["rect"])
+    assert np.abs(gpu["planes"] - o["planes"]).max() <= 1e-4   # FP32 planes, as above
