@@ -5,6 +5,10 @@
 // discrete Gaussian w[-r..r] (standard deviation sigma, in plane pixels) over
 // the rows, then over the columns, every RGBA channel, transparent zero
 // padding outside the plane, FP32 arithmetic, result stored in the plane type.
+//  k_filter_fused both passes in one walk, a cluster of CTAs per plane: every
+//                 texel is read once (and a halo) and written once; many
+//                 planes of up to 512 columns.
+//  The other planes take two passes:
 //  k_filter_rows  one CTA per (plane, row): the row is walked in segments;
 //                 each segment and its right halo are read into shared
 //                 memory, the left halo is the previous segment's tail of
@@ -20,6 +24,8 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include <type_traits>
+
 #include "lf_internal.cuh"
 
 namespace lf {
@@ -33,20 +39,32 @@ constexpr int kColLanes = 8;    // threads per column
 constexpr int kColBand = 32;    // output rows per step (>= 2 * kFilterMaxRadius: the carry never overlaps)
 static_assert(kColBand >= 2 * kFilterMaxRadius, "column carry would overlap");
 
+// a stored texel, and its FP32 channels
 template <int DT>
-__device__ __forceinline__ float4 ld(const void* p, size_t i)
+using Stored = std::conditional_t<DT == LF_F32, float4, std::conditional_t<DT == LF_U8, uint32_t, uint2>>;
+
+template <int DT>
+__device__ __forceinline__ float4 widen(Stored<DT> u)
 {
-    if (DT == LF_F32) return reinterpret_cast<const float4*>(p)[i];
-    if (DT == LF_U8) return u8_unpack(reinterpret_cast<const uint32_t*>(p)[i]);
-    const uint2 u = reinterpret_cast<const uint2*>(p)[i];
-    if (DT == LF_F16) {
+    if constexpr (DT == LF_F32) {
+        return u;
+    } else if constexpr (DT == LF_U8) {
+        return u8_unpack(u);
+    } else if constexpr (DT == LF_F16) {
         const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&u.x));
         const float2 b = __half22float2(*reinterpret_cast<const __half2*>(&u.y));
         return make_float4(a.x, a.y, b.x, b.y);
+    } else {
+        const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u.x));
+        const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u.y));
+        return make_float4(a.x, a.y, b.x, b.y);
     }
-    const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u.x));
-    const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u.y));
-    return make_float4(a.x, a.y, b.x, b.y);
+}
+
+template <int DT>
+__device__ __forceinline__ float4 ld(const void* p, size_t i)
+{
+    return widen<DT>(reinterpret_cast<const Stored<DT>*>(p)[i]);
 }
 
 template <int DT>
@@ -163,9 +181,166 @@ __global__ void __launch_bounds__(kColStrip* kColLanes) k_filter_cols(void* plan
     }
 }
 
+// ---------------------------------------------------------------------------
+// Both passes in one walk over a plane.
+// ---------------------------------------------------------------------------
+constexpr int kStrip = 64;            // columns per CTA
+constexpr int kBand = 16;             // rows per step
+constexpr int kFusedThreads = 256;    // 4 outputs per thread and pass: of one row, then of one column
+constexpr int kStripsMax = 8;         // CTAs per cluster (portable size)
+// One walk or two passes: a cluster takes a plane, so few planes leave SMs
+// idle and the two-pass kernels, with a CTA per row, win. 512^2 FP32, radius 3:
+// 24 planes 97 us (two passes 99), 32 99 (126), 64 164 (237); 256^2: 16 planes
+// 38 (36), 24 38 (44); 128^2: 32 planes 23 (23), 64 23 (33); FP16 64 planes of
+// 512^2 142 (208). Planes wider than eight strips don't fit a cluster.
+constexpr int kFusedPlanes = 32, kFusedCtas = 64;
+
+// the value that a store in the plane's type and a load back give
+template <int DT>
+__device__ __forceinline__ float4 as_stored(float4 v)
+{
+    if (DT == LF_F32) return v;
+    if (DT == LF_U8) return u8_unpack(u8_pack(v.x, v.y, v.z, v.w));
+    if (DT == LF_F16) {
+        const float2 a = __half22float2(__floats2half2_rn(v.x, v.y)), b = __half22float2(__floats2half2_rn(v.z, v.w));
+        return make_float4(a.x, a.y, b.x, b.y);
+    }
+    const float2 a = __bfloat1622float2(__floats2bfloat162_rn(v.x, v.y));
+    const float2 b = __bfloat1622float2(__floats2bfloat162_rn(v.z, v.w));
+    return make_float4(a.x, a.y, b.x, b.y);
+}
+
+// Four neighbouring outputs: out[q] = sum_t w[t] at(q + t), t = 0 .. 2 r in
+// order, each texel read once (2 r + 4 reads instead of 4 (2 r + 1)).
+template <typename At>
+__device__ __forceinline__ void slide4(const FilterParams& f, float4 (&out)[4], At at)
+{
+    const int n = 2 * f.radius;   // at least 2
+#pragma unroll
+    for (int q = 0; q < 4; ++q) out[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int t = 0; t < 3; ++t) {
+        const float4 v = at(t);
+#pragma unroll
+        for (int q = 0; q <= t; ++q) fma4(out[q], f.w[t - q], v);
+    }
+    for (int t = 3; t <= n; ++t) {
+        const float4 v = at(t);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) fma4(out[q], f.w[t - q], v);
+    }
+#pragma unroll
+    for (int t = 1; t <= 3; ++t) {
+        const float4 v = at(n + t);
+#pragma unroll
+        for (int q = t; q < 4; ++q)
+            if (n + t >= q) fma4(out[q], f.w[n + t - q], v);
+    }
+}
+
+// 16-byte slot of texel u of a row: eight lanes that read every fourth texel
+// hit eight different bank groups
+__device__ __forceinline__ int swz(int u) { return u ^ ((u >> 3) & 3); }
+
+// One cluster per plane, one CTA per strip of 64 columns, all of them walking
+// down in steps of 16 rows. A step puts the band's original texels (with r
+// columns on either side) into shared memory, filters its rows into a ring of
+// row-filtered rows, rounded to the plane's type as a stored row pass would
+// be, and filters the ring's columns into the output rows r above the band.
+// In place: a step writes only rows whose originals every CTA of the cluster
+// has read, its own and its neighbours' columns: the cluster barrier's arrive
+// follows the step's loads and its wait precedes the step's stores. The next
+// band's texels load into registers meanwhile.
+// The passes read 2 r + 4 texels of shared memory per four outputs (2 r + 1
+// per output in k_filter_rows and k_filter_cols). Bound by the latency of a
+// step at three or four CTAs per SM: 64 planes of 512^2 FP32, radius 3, take
+// 164 us (two passes 237; one read and one write of every texel at copy speed
+// 79).
+template <int DT>
+__global__ void __launch_bounds__(kFusedThreads, 4) k_filter_fused(void* planes, int W, int H, FilterParams f, int pitch,
+                                                                 int ring)
+{
+    extern __shared__ float4 fbuf[];
+    float4* raw = fbuf;                        // [kBand][pitch]
+    float4* rows = fbuf + kBand * pitch;       // [ring][kStrip], row y at y & (ring - 1)
+    // texels of a band: thread t loads columns t % 16 + 16 q of row t / 16
+    constexpr int kLoads = (kStrip + 2 * kFilterMaxRadius) / 16;
+    static_assert(kFusedThreads == 16 * kBand, "sixteen threads per row of a band");
+    const int tid = threadIdx.x, r = f.radius, lrow = tid / 16, lu = tid % 16;
+    const int x0 = (int)blockIdx.x * kStrip, span = kStrip + 2 * r;
+    const size_t plane = (size_t)blockIdx.y * (size_t)W * H;
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int i = tid; i < ring * kStrip; i += kFusedThreads) rows[i] = zero;   // rows above the plane
+    Stored<DT> next[kLoads];   // as stored: a conversion would wait for the load
+    auto load = [&](int y) {
+        const Stored<DT>* src = reinterpret_cast<const Stored<DT>*>(planes) + (plane + (size_t)y * W);
+#pragma unroll
+        for (int q = 0; q < kLoads; ++q) {
+            const int x = x0 - r + lu + 16 * q;
+            next[q] = Stored<DT>{};   // all types: 0
+            if (y < H && lu + 16 * q < span && x >= 0 && x < W) next[q] = src[x];
+        }
+    };
+    load(lrow);
+    for (int y0 = 0; y0 < H + r; y0 += kBand) {
+#pragma unroll
+        for (int q = 0; q < kLoads; ++q)
+            if (lu + 16 * q < span) raw[lrow * pitch + swz(lu + 16 * q)] = widen<DT>(next[q]);
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+        __syncthreads();
+        if (y0 + kBand < H + r) load(y0 + kBand + lrow);
+        float4 out[4];
+        {
+            const int row = tid / (kStrip / 4), c = tid % (kStrip / 4) * 4;
+            const float4* src = raw + row * pitch;
+            slide4(f, out, [&](int t) { return src[swz(c + t)]; });
+            float4* dst = rows + ((y0 + row) & (ring - 1)) * kStrip;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) dst[swz(c + q)] = as_stored<DT>(out[q]);
+        }
+        __syncthreads();
+        {
+            const int c = tid % kStrip, y = y0 - r + tid / kStrip * 4;   // first output row
+            slide4(f, out, [&](int t) { return rows[((y - r + t) & (ring - 1)) * kStrip + swz(c)]; });
+            asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (y + q >= 0 && y + q < H && x0 + c < W) st<DT>(planes, plane + (size_t)(y + q) * W + x0 + c, out[q]);
+        }
+    }
+}
+
+template <int DT>
+void launch_fused(void* planes, int N, int W, int H, const FilterParams& f, cudaStream_t s)
+{
+    const int strips = (W + kStrip - 1) / kStrip;
+    const int pitch = (kStrip + 2 * f.radius + 31) / 32 * 32, ring = kBand + 2 * f.radius <= 32 ? 32 : 64;
+    const size_t smem = sizeof(float4) * (size_t)(kBand * pitch + ring * kStrip);
+    auto kern = k_filter_fused<DT>;
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)strips, (unsigned)N);
+    cfg.blockDim = dim3(kFusedThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = (unsigned)strips;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kern, planes, W, H, f, pitch, ring);
+    note_launches(1);
+}
+
 template <int DT>
 void launch_filter_t(void* planes, int N, int W, int H, const FilterParams& f, cudaStream_t s)
 {
+    const int strips = (W + kStrip - 1) / kStrip;
+    if (f.radius >= 1 && strips <= kStripsMax && N >= kFusedPlanes && N <= 65535 && strips * N >= kFusedCtas) {
+        launch_fused<DT>(planes, N, W, H, f, s);
+        return;
+    }
     k_filter_rows<DT><<<(unsigned)((size_t)N * H), kRowThreads, sizeof(float4) * (kSeg + 2 * f.radius), s>>>(
         planes, W, H, f);
     const dim3 grid((unsigned)((W + kColStrip - 1) / kColStrip), (unsigned)N);
