@@ -224,7 +224,8 @@ lf_status lf_build_mpi_voxels(const lf_voxels* v, const lf_ref_camera* ref, int3
 
 /* Synchronises with the stream the last build on ws was enqueued on and
  * returns LF_ERR_OVERFLOW if its tile list exceeded the capacity (the planes
- * are then all zero); *needed (host, may be NULL) receives the pair count
+ * are then all zero), LF_ERR_TIMEOUT if a bounded device wait of the build
+ * gave up (the planes are then not valid); *needed (host, may be NULL) receives the pair count
  * and *culled_in (host, may be NULL) the number M of primitives kept. */
 lf_status lf_mpi_status(const void* ws, int64_t* needed, int64_t* culled_in);
 
@@ -384,10 +385,9 @@ lf_status lf_build_mpi_backward_voxels(const lf_voxels* v, const lf_ref_camera* 
 /*
  * Several G2LF scenes of uneven sizes, view counts, resolutions and N
  * rendered together: each scene's build runs up to its tile lists, then ONE
- * persistent raster launch covers the (tile, chunk) items of every scene and
- * ONE persistent staged-composite launch covers the (chunk group, view
- * group, row band, column tile) items of every scene, CTAs pulling items
- * from a global counter; or (schedule 2) every scene's single-scene pipeline
+ * raster launch covers the (tile, chunk) lists of every scene and ONE
+ * composite launch covers the (chunk group, view group, row band, column
+ * tile) items of every scene, one CTA per item; or (schedule 2) every scene's single-scene pipeline
  * runs on a stream of its own, all in parallel. With chunk groups G > 1 a
  * scene's non-empty planes are cut into G contiguous shares composited
  * separately into partial (Q, T) per view pixel and then composed front to
@@ -421,16 +421,16 @@ typedef struct {
 } lf_batch_scene;
 
 /* Launch plan of a batch:
- *  views_per_thread  composite views per thread: 3, 5, 9 or 15 (15: one
- *                    CTA per SM, the others two);
- *  tile_x            composite CTA tile width (columns): 128, 256 or 512
- *                    (the tile is tile_x x 512/tile_x pixels);
+ *  views_per_thread  composite views per thread: 3, 5, 9 or 15;
+ *  tile_x            128, 256 or 512: a composite CTA's tile is at most
+ *                    tile_x / 4 columns of its 128 pixels wide (each scene
+ *                    takes the best width up to that);
  *  chunk_groups      1, 2 or 4: the contiguous shares of every scene's
  *                    non-empty planes that are composited as separate items
  *                    and composed in order (partial buffers in the batch
  *                    workspace: lf_batch_plan_workspace_size);
  *  schedule          0: items in scene order; 1: largest scenes first;
- *                    2: no persistent launches -- every scene's own
+ *                    2: no common launches -- every scene's own
  *                    lf_build_mpi_gaussians + lf_composite on a stream of its
  *                    own, forked from and joined back into the caller's
  *                    stream (the other fields are then unused). */
@@ -463,9 +463,8 @@ size_t lf_batch_plan_workspace_size(const lf_batch* b, const lf_batch_plan* plan
  * a plan change; not during capture. */
 lf_status lf_batch_prepare(lf_batch* b, const lf_batch_plan* plan, void* ws, size_t ws_bytes, cudaStream_t stream);
 
-/* Enqueues one frame of the whole batch on stream (builds, persistent
- * raster, coefficient tables, persistent composite). No host
- * synchronisation; may be captured. */
+/* Enqueues one frame of the whole batch on stream (builds, raster,
+ * coefficient tables, composite). No host synchronisation; may be captured. */
 lf_status lf_batch_render(lf_batch* b, cudaStream_t stream);
 
 /* Captures lf_batch_render on stream (which must not be the legacy default
@@ -485,8 +484,8 @@ lf_status lf_batch_autotune(lf_batch* b, void* ws, size_t ws_bytes, int32_t reps
                             lf_batch_plan* best, float* best_ms);
 
 /* Synchronises stream and returns LF_ERR_OVERFLOW if a scene's tile list
- * overflowed its capacity, LF_ERR_TIMEOUT if a bounded wait of the
- * composite gave up, else LF_OK. */
+ * overflowed its capacity, LF_ERR_TIMEOUT if a bounded wait of a build or
+ * of the composite gave up, else LF_OK. */
 lf_status lf_batch_status(lf_batch* b, cudaStream_t stream);
 
 /* Frees the batch object and its graph (device memory stays the caller's). */
@@ -499,8 +498,8 @@ int64_t lf_launch_count(void);
 
 /* Turns stage tracing on or off for calls made from this thread: while on,
  * every pipeline stage of lf_build_mpi_* and lf_composite (project,
- * depth_sort, bin, duplicate, tile_sort, ranges, raster_*, comp_coeffs,
- * composite) is bracketed by a CUDA event pair recorded on the call's stream.
+ * depth_sort, bin: chunks and tile pairs, tile_lists: their sort and ranges,
+ * raster_*, comp_coeffs, composite) is bracketed by a CUDA event pair recorded on the call's stream.
  * Always returns LF_OK. */
 lf_status lf_trace_enable(int32_t on);
 
@@ -514,10 +513,10 @@ int32_t lf_trace_collect(char* names, double* total_ms, int64_t* launches, int32
 /* ---- failure detection ----------------------------------------------------- */
 
 /* Every device-side wait of the library (the staged composite's mbarrier
- * waits) is bounded: after 2 s of wall time it gives up, the kernel sets the
- * call's error word and returns, and lf_composite_status / lf_batch_status
- * report LF_ERR_TIMEOUT;
- * the CUDA context stays usable. This self-test exercises that path without
+ * waits, the build's waits for the sums of earlier blocks) is bounded: it
+ * gives up after 2 s of wall time or a number of tries, the kernel sets the
+ * call's error word and returns, and lf_composite_status / lf_mpi_status /
+ * lf_batch_status report LF_ERR_TIMEOUT; the CUDA context stays usable. This self-test exercises that path without
  * a fault: one thread waits, with a limit of limit_ms (1..10000)
  * milliseconds, on a shared-memory mbarrier that nothing arrives on.
  * Synchronises the stream; returns LF_ERR_TIMEOUT when the wait gave up as

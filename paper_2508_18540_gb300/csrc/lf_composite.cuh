@@ -306,28 +306,6 @@ __device__ __forceinline__ bool produce(const CompParams& p, const CompGeom& G, 
         if (!mbar_wait_bounded(sm.empty + 8 * ring.st, ring.ph ^ 1u)) return 2;
         return EARLY && *reinterpret_cast<volatile int*>(sm.sat) == kWarps ? 1 : 0;
     };
-    // bulk copies of one step into sa (its copy record c)
-    auto stage_step = [&](int i, uint32_t sa, float4 c, uint32_t full) {
-        if (VG > 1) bulk_copy_g2s(sa, blk + (size_t)entry(i) * CW + 4, 4u * KV, full);
-        const uint32_t bytes = __float_as_uint(c.z);
-        if (!bytes) return;
-        const char* src = planes + ((unsigned long long)__float_as_uint(c.y) << 32 | __float_as_uint(c.x));
-        uint32_t rows = __float_as_uint(c.w), dst = sa + G.hdr_bytes;
-        const size_t pitch = (size_t)p.W * TB;
-        if (G.BY == 1) {
-#pragma unroll
-            for (int t = 0; t < RPY; ++t)
-                if (rows & (1u << t)) bulk_copy_g2s(dst + (uint32_t)t * G.win_bytes, src + t * pitch, bytes, full);
-            return;
-        }
-        const float4 B = lds_f4(sm.desc + (uint32_t)(i & (kDescs - 1)) * DB + 16);
-        const int iy0 = plane_index(p.P_s, Y0, B.x, B.y);
-        for (; rows; rows &= rows - 1) {
-            const int r = __ffs(rows) - 1;
-            const int iy = plane_index(p.P_s, Y0 + r / RPY, B.x, B.y) + r % RPY;
-            bulk_copy_g2s(dst + (uint32_t)r * G.win_bytes, src + (ptrdiff_t)(iy - iy0) * (ptrdiff_t)pitch, bytes, full);
-        }
-    };
     fetch(lane);
     for (int i0 = 0; i0 < n; i0 += 32) {
         const float4 hd = nh;
@@ -380,41 +358,51 @@ __device__ __forceinline__ bool produce(const CompParams& p, const CompGeom& G, 
         __syncwarp();
         const int cnt = min(32, n - i0);
         int stop = 0;
+        const int R = G.BY * RPY, u = lane >> 4, j = lane & 15;
         if (G.bulk) {
-            if (lane == 0) {
-                for (int e = 0; e < cnt; e += kPair) {
-                    const int i = i0 + e;
-                    const uint32_t full = sm.full + 8 * ring.st;
-                    if ((stop = acquire(i)) != 0) {
-                        if (stop == 1) {
-                            *reinterpret_cast<volatile int*>(sm.end) = i;
-                            mbar_arrive(full);
-                            ring.next(G.stages);
-                        }
-                        break;
+            // lane 16 u + j copies row j of the stage's step u, j = R the
+            // step's h: issued by one lane, the copies of four-row tiles took
+            // half a microsecond a step, more than a small grid's blending
+            for (int e = 0; e < cnt; e += kPair) {
+                const int i = i0 + e;
+                const uint32_t full = sm.full + 8 * ring.st;
+                if (lane == 0) stop = acquire(i);
+                __syncwarp();
+                stop = __shfl_sync(0xffffffffu, stop, 0);
+                if (stop) {
+                    if (stop == 1 && lane == 0) {
+                        *reinterpret_cast<volatile int*>(sm.end) = i;
+                        mbar_arrive(full);
                     }
-                    uint32_t sa = sm.stages + (uint32_t)ring.st * G.stage_bytes;
-                    uint32_t c = sm.copies + 16 * (uint32_t)(i & (kDescs - 1));
-                    const bool two = e + 1 < cnt;
-                    const float4 c0 = lds_f4(c), c1 = lds_f4(c + 16);   // (an unused second record is not read further)
-                    const uint32_t b0 = __float_as_uint(c0.z), b1 = two ? __float_as_uint(c1.z) : 0u;
-                    if (!BILINEAR) {
-                        // the zero texel behind the rows' windows (read in mode kBorder)
-                        for (int r = 0; r < G.BY; ++r) {
-                            sts_f4(sa + G.hdr_bytes + (uint32_t)r * G.win_bytes + b0, make_float4(0.f, 0.f, 0.f, 0.f));
-                            sts_f4(sa + G.plane_bytes + G.hdr_bytes + (uint32_t)r * G.win_bytes + b1,
-                                   make_float4(0.f, 0.f, 0.f, 0.f));
-                        }
-                    }
-                    fence_proxy_async();
-                    mbar_arrive_expect_tx(full, (two ? 8u : 4u) * KV + (uint32_t)__popc(__float_as_uint(c0.w)) * b0 +
-                                                    (uint32_t)__popc(__float_as_uint(c1.w)) * b1);
-                    stage_step(i, sa, c0, full);
-                    if (two) stage_step(i + 1, sa + G.plane_bytes, c1, full);
-                    ring.next(G.stages);
+                    if (stop == 1) ring.next(G.stages);
+                    break;
                 }
+                const bool has = e + u < cnt;
+                const uint32_t slot = (uint32_t)((i + u) & (kDescs - 1));
+                const uint32_t sa = sm.stages + (uint32_t)ring.st * G.stage_bytes + (u ? G.plane_bytes : 0u);
+                const uint32_t dst = sa + G.hdr_bytes + (uint32_t)j * G.win_bytes;
+                const float4 c = has ? lds_f4(sm.copies + 16 * slot) : make_float4(0.f, 0.f, 0.f, 0.f);
+                const uint32_t bytes = __float_as_uint(c.z), rows = __float_as_uint(c.w);
+                // the zero texel behind the row's window (read in mode kBorder)
+                if (!BILINEAR && has && j < R) sts_f4(dst + bytes, make_float4(0.f, 0.f, 0.f, 0.f));
+                fence_proxy_async();
+                const uint32_t tx = has ? 4u * KV + (uint32_t)__popc(rows) * bytes : 0u;
+                const uint32_t both = tx + __shfl_xor_sync(0xffffffffu, tx, 16);
+                __syncwarp();   // lane 0's arrival orders the zero texels too
+                if (lane == 0) mbar_arrive_expect_tx(full, both);
+                __syncwarp();
+                if (has && j == R && VG > 1) bulk_copy_g2s(sa, blk + (size_t)entry(i + u) * CW + 4, 4u * KV, full);
+                if (bytes && j < R && ((rows >> j) & 1u)) {
+                    const char* src = planes + ((unsigned long long)__float_as_uint(c.y) << 32 | __float_as_uint(c.x));
+                    int down = j % RPY;
+                    if (j >= RPY) {
+                        const float4 B = lds_f4(sm.desc + slot * DB + 16);
+                        down += plane_index(p.P_s, Y0 + j / RPY, B.x, B.y) - plane_index(p.P_s, Y0, B.x, B.y);
+                    }
+                    bulk_copy_g2s(dst, src + (ptrdiff_t)down * (ptrdiff_t)((size_t)p.W * TB), bytes, full);
+                }
+                ring.next(G.stages);
             }
-            stop = __shfl_sync(0xffffffffu, stop, 0);
         } else {
             for (int e = 0; e < cnt; e += kPair) {
                 const int i = i0 + e;
@@ -430,24 +418,38 @@ __device__ __forceinline__ bool produce(const CompParams& p, const CompGeom& G, 
                     }
                     break;
                 }
-                uint32_t sa = sm.stages + (uint32_t)ring.st * G.stage_bytes;
-                for (int u = 0; u < min(kPair, cnt - e); ++u, sa += G.plane_bytes) {
-                    const uint32_t slot = (uint32_t)((i + u) & (kDescs - 1));
-                    const float4 c4 = lds_f4(sm.copies + 16 * slot), B = lds_f4(sm.desc + slot * DB + 16);
-                    if (VG > 1 && lane < KV / 4)
-                        cp_async<16>(sa + 16u * (uint32_t)lane, blk + (size_t)entry(i + u) * CW + 4 + 4 * lane);
-                    const char* base = planes + ((unsigned long long)__float_as_uint(c4.y) << 32 | __float_as_uint(c4.x));
-                    const int texels = (int)(__float_as_uint(c4.z) / TB);
-                    const int iy0 = plane_index(p.P_s, Y0, B.x, B.y);
-                    for (uint32_t rows = texels ? __float_as_uint(c4.w) : 0u; rows; rows &= rows - 1) {
-                        const int r = __ffs(rows) - 1;
-                        const int iy = plane_index(p.P_s, Y0 + r / RPY, B.x, B.y) + r % RPY;
-                        const char* src = base + (ptrdiff_t)(iy - iy0) * (ptrdiff_t)((size_t)p.W * TB);
-                        const uint32_t dst = sa + G.hdr_bytes + (uint32_t)r * G.win_bytes;
-                        for (int c = lane; c < texels; c += 32) cp_async<TB>(dst + (uint32_t)c * TB, src + (size_t)c * TB);
-                        // the zero texel behind the window
-                        if (!BILINEAR && lane < TB / 4) sts_f1(dst + (uint32_t)texels * TB + 4u * (uint32_t)lane, 0.f);
+                // lane 16 u + j finds row j of step u, then all lanes copy row by row
+                const bool has = e + u < cnt;
+                const uint32_t slot = (uint32_t)((i + u) & (kDescs - 1));
+                const uint32_t sa = sm.stages + (uint32_t)ring.st * G.stage_bytes + (u ? G.plane_bytes : 0u);
+                const uint32_t dst = sa + G.hdr_bytes + (uint32_t)j * G.win_bytes;
+                const float4 c4 = has ? lds_f4(sm.copies + 16 * slot) : make_float4(0.f, 0.f, 0.f, 0.f);
+                if (VG > 1 && has && j < KV / 4)
+                    cp_async<16>(sa + 16u * (uint32_t)j, blk + (size_t)entry(i + u) * CW + 4 + 4 * j);
+                const int texels = (int)(__float_as_uint(c4.z) / TB);
+                const bool on = texels && j < R && ((__float_as_uint(c4.w) >> j) & 1u);
+                unsigned long long src = 0;
+                if (on) {
+                    int down = j % RPY;
+                    if (j >= RPY) {
+                        const float4 B = lds_f4(sm.desc + slot * DB + 16);
+                        down += plane_index(p.P_s, Y0 + j / RPY, B.x, B.y) - plane_index(p.P_s, Y0, B.x, B.y);
                     }
+                    src = (unsigned long long)planes +
+                          ((unsigned long long)__float_as_uint(c4.y) << 32 | __float_as_uint(c4.x)) +
+                          (unsigned long long)((long long)down * (long long)((size_t)p.W * TB));
+                    // the zero texel behind the window
+                    if (!BILINEAR) {
+#pragma unroll
+                        for (int t = 0; t < TB / 4; ++t) sts_f1(dst + (uint32_t)texels * TB + 4u * t, 0.f);
+                    }
+                }
+                for (uint32_t m = __ballot_sync(0xffffffffu, on); m; m &= m - 1) {
+                    const int l = __ffs(m) - 1;
+                    const char* from = reinterpret_cast<const char*>(__shfl_sync(0xffffffffu, src, l));
+                    const uint32_t to = __shfl_sync(0xffffffffu, dst, l);
+                    const int n_tex = __shfl_sync(0xffffffffu, texels, l);
+                    for (int c = lane; c < n_tex; c += 32) cp_async<TB>(to + (uint32_t)c * TB, from + (size_t)c * TB);
                 }
                 cp_async_arrive(full);
                 __syncwarp();   // lane 0's arrival orders the zero texels too
