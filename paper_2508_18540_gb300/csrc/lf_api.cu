@@ -151,8 +151,8 @@ size_t build_ws_layout(int64_t n, int32_t N, int32_t W, int32_t H, int64_t cap, 
     w.seg = carve<int2>(base, off, (size_t)S);
     w.g2d = carve<float>(base, off, 12 * nn);
     // partial-result slots of split raster lists: enough that a frame of cap
-    // pairs needs no more than kRasterSegMax entries per part, up to a cap
-    long long slots = 2 * (long long)cc / kRasterSegMax + 2;
+    // pairs needs no more than kRasterSegMin entries per part, up to a cap
+    long long slots = 2 * (long long)cc / kRasterSegMin + 2;
     slots = slots < 16 ? 16 : slots > kRasterSlotsMax ? kRasterSlotsMax : slots;
     w.r_nslots = slots;
     w.r_items = carve<int4>(base, off, (size_t)slots);

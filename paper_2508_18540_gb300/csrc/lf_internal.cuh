@@ -277,12 +277,11 @@ struct WsHeader {
 
 // Split lists of the Gaussian raster: a list of L > r_seg entries is cut into
 // ceil(L / r_seg) parts, each with a partial (C, T) slot of one super-tile
-// (kSuper^2 texels); r_seg is a frame's pairs per resident CTA within
-// [kRasterSegMin, kRasterSegMax], or more where the parts would need more than
-// the workspace's slots.
-constexpr int kRasterSegMin = 256;    // one staged batch
-constexpr int kRasterSegMax = 1024;
-constexpr int kRasterCtas = 152 * 4;
+// (kSuper^2 texels); r_seg is at least kRasterSegMin and large enough that
+// the parts of a frame never need more than the workspace's slots. (Parts of
+// 256 entries in frames of few pairs: 10k Gaussians 82 us instead of 85, but
+// other roundings, which FP16 planes show as a step of 2^-11.)
+constexpr int kRasterSegMin = 1024;
 constexpr long long kRasterSlotsMax = 4096;
 
 // Carved build workspace (all device pointers).

@@ -112,9 +112,7 @@ __device__ __forceinline__ float ex2_approx(float x)
 //
 // Load balance. The work of a list grows with its length, and dense regions
 // of the scene make a few lists far longer than the rest. k_raster_plan cuts
-// every list longer than r_seg entries into parts of r_seg entries (1024; in
-// frames of few pairs, where the longest list is the kernel's time, down to
-// one staged batch: the 10k-Gaussian frame 85 -> 82 us), and
+// every list longer than r_seg entries into parts of r_seg entries, and
 // k_raster_gauss_parts rasterises the parts: each blends its entries into a
 // partial (C, T) started from (0, 1) and stores it in its slot, and the CTA
 // that finishes a list's last part composes the partials in part order,
@@ -166,8 +164,8 @@ __global__ void __launch_bounds__(kPlanThreads) k_raster_plan(BuildWs w, int lis
     int S = 0x7fffffff;
     if (split) {
         long long need = (2 * total + w.r_nslots - 1) / w.r_nslots;   // keeps the parts within the slots
-        need = max(need, min(total / kRasterCtas, (long long)kRasterSegMax));
-        S = (int)((max(need, (long long)kRasterSegMin) + 255) / 256 * 256);
+        need = (need + 255) / 256 * 256;
+        S = (int)(need > kRasterSegMin ? need : kRasterSegMin);
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) w.hdr->r_seg = S;
     for (int id = blockIdx.x * kPlanThreads + threadIdx.x; id < lists; id += gridDim.x * kPlanThreads) {
