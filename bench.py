@@ -637,7 +637,7 @@ def run_batched(args, dev):
             "views_per_s": round(views * 1000.0 / g_ms, 1), "kernels_per_frame": int(launches),
             "one_by_one_ms_per_frame": round(s_ms, 3),
             "chunk_groups_ms_per_frame": by_groups,
-            "chunk_groups_note": "persistent schedule (tuned composite layout), plain launches, L2 flushed"}
+            "chunk_groups_note": "common launches (tuned composite layout), plain launches, L2 flushed"}
 
 
 def run_sweeps(args, dev):
