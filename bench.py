@@ -61,14 +61,13 @@ def _config(extra=None):
 
 
 # DRAM bytes (read + write) per launch from one ncu capture of the f32 frame
-# (profiles/k_*_g2lf_display_1M_512px_N64_45v.md), valid only while the
+# (profiles/*_g2lf_display_1M_512px_N64_45v.md), valid only while the
 # kernel's sources (their code, comments aside) hash to the value recorded
 # with them.
 NCU_TRAFFIC = {
     # the raster stage's two kernels: the parts of split lists and the lists
-    "raster_gaussians": (11_979_008 + 0 + 71_470_848 + 204_340_480, ("lf_raster.cu", "lf_internal.cuh"),
-                         "3e0cef0f8f9d1f2b"),
-    "composite": (252_981_760 + 156_500_736, ("lf_composite.cu", "lf_internal.cuh"), "d93198e445d327bc"),
+    "raster_gaussians": (7_750_144 + 276_028_928, ("lf_raster.cu", "lf_internal.cuh"), "aa576407fcce1e36"),
+    "composite": (366_265_344, ("lf_composite.cuh", "lf_composite.cu", "lf_internal.cuh"), "8a4945b15aa93f29"),
 }
 
 
