@@ -611,12 +611,12 @@ class HostPipeline:
 
 
 # ---------------------------------------------------------------------------
-# batching: several scenes, persistent launches, CUDA graph, autotuner
+# batching: several scenes, common launches, CUDA graph, autotuner
 # ---------------------------------------------------------------------------
 
 class BatchRenderer:
     """Several Gaussian scenes rendered as one batch (lf_batch_*): per-scene
-    builds, one persistent raster and one persistent composite launch over
+    builds, one raster and one composite launch over
     every scene's work items; optionally captured once into a CUDA graph.
     workloads: objects with scene, camera, display, views, N, binning.
     Scene data is copied to the device once (update it in place through

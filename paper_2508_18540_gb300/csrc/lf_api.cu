@@ -341,7 +341,7 @@ static lf_status check_composite_args(const lf_planes* planes, const lf_ref_came
 }
 
 // The build pipeline. With prefix_only the raster is left to the caller
-// (the batched persistent raster), which gets the carved workspace and the
+// (the batched raster), which gets the carved workspace and the
 // sorted tile-list ranks back.
 template <typename Launch>
 static lf_status build_common(int64_t n, const lf_ref_camera* ref, int32_t N, int32_t binning, void* ws,

@@ -1,5 +1,5 @@
 // lf_batch.cu -- several G2LF scenes in one frame: per-scene builds up to the
-// tile lists, then one persistent raster launch and one persistent staged
+// tile lists, then one raster launch and one staged
 // composite launch over the work items of every scene (schedules 0 and 1),
 // or every scene's own pipeline on a stream of its own, forked from and
 // joined back into the caller's stream (schedule 2); CUDA-graph capture of

@@ -394,7 +394,7 @@ void launch_raster_gaussians(const BuildWs& ws, const RasterParams& p, const uin
 void launch_raster_voxels(const BuildWs& ws, const RasterParams& p, const uint32_t* ranks, void* planes,
                           cudaStream_t s);
 
-// batched (several scenes, one persistent launch): per-scene item table
+// batched (several scenes, one launch): per-scene item table
 struct RasterScene {
     BuildWs w;
     RasterParams p;

@@ -1,4 +1,4 @@
-"""The paired Gaussian raster at its edges: list lengths around the parts that
+"""The paired Gaussian raster at its edges: list lengths around a staged batch and the parts that
 long lists are cut into, planes that end inside a block of 8 x 8 pixels, and
 colours that are not finite."""
 import numpy as np
