@@ -525,6 +525,17 @@ int32_t lf_trace_collect(char* names, double* total_ms, int64_t* launches, int32
  * variable). */
 lf_status lf_selftest_bounded_wait(int32_t limit_ms, cudaStream_t stream);
 
+/* The other waits: lf_build_mpi_gaussians with every wait of a block for the
+ * sums of earlier blocks giving up at its first poll (no fault, no delay).
+ * Same arguments, checks and workspace; enqueued on stream. With more
+ * primitives than one block takes (2048 in the depth sort, 256 in the binning),
+ * or more (primitive, 32 x 32 super-tile) pairs than one block sorts (2048),
+ * lf_mpi_status(ws) then returns LF_ERR_TIMEOUT, the planes are all zero with
+ * no members, and the adjoints on ws give zero gradients; the next build on ws
+ * is a normal one. */
+lf_status lf_selftest_build_waits(const lf_gaussians* g, const lf_ref_camera* ref, int32_t N, int32_t binning,
+                                  void* ws, size_t ws_bytes, lf_planes* out, cudaStream_t stream);
+
 /* ---- misc --------------------------------------------------------------- */
 
 /* Thread-local description of the last error on this thread ("" if none). */

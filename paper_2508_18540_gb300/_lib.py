@@ -131,6 +131,8 @@ SIGNATURES = [
     ("lf_batch_status", ctypes.c_int, [_P, _P]),
     ("lf_batch_destroy", ctypes.c_int, [_P]),
     ("lf_selftest_bounded_wait", ctypes.c_int, [_I32, _P]),
+    ("lf_selftest_build_waits", ctypes.c_int, [ctypes.POINTER(LfGaussians), ctypes.POINTER(LfRefCamera), _I32, _I32,
+                                               _P, ctypes.c_size_t, ctypes.POINTER(LfPlanes), _P]),
     ("lf_composite_status", ctypes.c_int, [_I32, ctypes.POINTER(LfViewSet), _P, _P]),
     ("lf_launch_count", _I64, []),
     ("lf_trace_enable", ctypes.c_int, [_I32]),

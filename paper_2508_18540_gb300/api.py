@@ -726,6 +726,16 @@ def lf_selftest_bounded_wait(limit_ms: int = 50, stream=None) -> int:
     return int(load().lf_selftest_bounded_wait(int(limit_ms), _stream_ptr(stream)))
 
 
+def lf_selftest_build_waits(g: DeviceGaussians, ref: L.LfRefCamera, N: int, binning: str, ws: torch.Tensor,
+                            planes: Planes, stream=None):
+    """lf_build_mpi_gaussians whose waits for earlier blocks' sums give up at
+    their first poll; lf_mpi_status then reports LF_ERR_TIMEOUT (asynchronous)."""
+    gs = g.c_struct()
+    ps = planes.c_struct()
+    check(load().lf_selftest_build_waits(ctypes.byref(gs), ctypes.byref(ref), int(N), BINNING[binning], _ptr(ws),
+                                         ws.numel(), ctypes.byref(ps), _stream_ptr(stream)))
+
+
 def lf_trace_enable(on: bool):
     check(load().lf_trace_enable(int(bool(on))))
 

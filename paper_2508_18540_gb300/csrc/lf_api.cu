@@ -160,6 +160,7 @@ size_t build_ws_layout(int64_t n, int32_t N, int32_t W, int32_t H, int64_t cap, 
     w.r_part = carve<float4>(base, off, (size_t)slots * kSuper * kSuper);
     w.bytes = align_up(off, 256);
     w.nb_dup = nbd;
+    w.look_tries = kLookbackTries;
     if (o) *o = w;
     return w.bytes;
 }
@@ -347,7 +348,7 @@ template <typename Launch>
 static lf_status build_common(int64_t n, const lf_ref_camera* ref, int32_t N, int32_t binning, void* ws,
                               size_t ws_bytes, lf_planes* out, cudaStream_t stream, int kind, Launch project,
                               const void* raster_arg, bool prefix_only = false, BuildWs* w_out = nullptr,
-                              const uint32_t** ranks_out = nullptr)
+                              const uint32_t** ranks_out = nullptr, int look_tries = kLookbackTries)
 {
     lf_status st = check_ref(ref);
     if (st != LF_OK) return st;
@@ -371,6 +372,7 @@ static lf_status build_common(int64_t n, const lf_ref_camera* ref, int32_t N, in
     }
     BuildWs w;
     build_ws_layout(n, N, ref->W, ref->H, cap, ws, &w);
+    w.look_tries = look_tries;
 
     {
         std::lock_guard<std::mutex> lk(g_ws_mu);
@@ -611,8 +613,9 @@ size_t lf_build_mpi_workspace_size(const lf_ref_camera* ref, int64_t n, int32_t 
     return build_ws_layout(n, N, ref->W, ref->H, dup_capacity, nullptr, nullptr);
 }
 
-lf_status lf_build_mpi_gaussians(const lf_gaussians* g, const lf_ref_camera* ref, int32_t N, int32_t binning,
-                                 void* ws, size_t ws_bytes, lf_planes* out, cudaStream_t stream)
+// look_tries: limit of the build's waits for earlier blocks' sums
+static lf_status build_gaussians(const lf_gaussians* g, const lf_ref_camera* ref, int32_t N, int32_t binning, void* ws,
+                                 size_t ws_bytes, lf_planes* out, cudaStream_t stream, int look_tries)
 {
     if (!g) return fail(LF_ERR_INVALID_ARG, "gaussians is NULL");
     if (g->n > 0 && (!g->means || !g->scales || !g->quats || !g->opacity || !g->rgb))
@@ -621,7 +624,20 @@ lf_status lf_build_mpi_gaussians(const lf_gaussians* g, const lf_ref_camera* ref
     auto project = [&](const ProjParams& pp, const BuildWs& w, cudaStream_t s) {
         launch_project_gaussians(gc, pp, w, out->rect, out->chunk, s);
     };
-    return build_common(g->n, ref, N, binning, ws, ws_bytes, out, stream, 0, project, &gc);
+    return build_common(g->n, ref, N, binning, ws, ws_bytes, out, stream, 0, project, &gc, false, nullptr, nullptr,
+                        look_tries);
+}
+
+lf_status lf_build_mpi_gaussians(const lf_gaussians* g, const lf_ref_camera* ref, int32_t N, int32_t binning,
+                                 void* ws, size_t ws_bytes, lf_planes* out, cudaStream_t stream)
+{
+    return build_gaussians(g, ref, N, binning, ws, ws_bytes, out, stream, kLookbackTries);
+}
+
+lf_status lf_selftest_build_waits(const lf_gaussians* g, const lf_ref_camera* ref, int32_t N, int32_t binning,
+                                  void* ws, size_t ws_bytes, lf_planes* out, cudaStream_t stream)
+{
+    return build_gaussians(g, ref, N, binning, ws, ws_bytes, out, stream, -1);
 }
 
 lf_status lf_build_mpi_voxels(const lf_voxels* v, const lf_ref_camera* ref, int32_t N, int32_t binning, void* ws,

@@ -251,7 +251,7 @@ __global__ void __launch_bounds__(kT, EMIT ? 4 : 6) k_bin_emit(BuildWs w, BinPar
             base += x;
             t -= use;
             idle = use ? 0 : idle + 1;
-            if (idle > kLookbackTries) {
+            if (idle > w.look_tries) {
                 if (lane == 0) atomicExch(&w.hdr->timeout, 1);
                 done = true;
             }

@@ -78,8 +78,9 @@ inline void launch_overlapped(void (*kern)(KArgs...), dim3 grid, dim3 block, siz
 #endif
 
 // ---- mbarriers with bounded waits (shared by the staged kernels) ---------
-// Every device-side wait of the library gives up after about kWaitLimitNs of
-// wall time or kSpinLimit tries; its caller then records an error word.
+// Every wait on an mbarrier gives up after about kWaitLimitNs of wall time or
+// kSpinLimit tries; its caller then records an error word. (The build's waits
+// for earlier blocks' sums have a limit of their own, kLookbackTries.)
 constexpr long long kSpinLimit = 1ll << 26;
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;   // 2 s: a wait that long has failed
 #ifdef __CUDACC__
@@ -148,7 +149,12 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity)
 // ---- decoupled look-back ---------------------------------------------------
 // A block publishes its own sum (kSumOwn), then, once it has added up the
 // blocks before it, the sum up to and with itself (kSumAll), in one 64-bit
-// word: two flag bits over a 62-bit count.
+// word: two flag bits over a 62-bit count. A block that polls
+// BuildWs::look_tries times without progress sets WsHeader::timeout and goes on
+// with the sum it has. That sum is never above the true one, so its own writes
+// stay in range, but the order it leaves is not valid: entries are lost, and the
+// places they would have taken hold whatever was there before. So every later
+// kernel of the build and the adjoints start by looking at the flag.
 #ifdef __CUDACC__
 constexpr unsigned long long kSumOwn = 1ull << 62, kSumAll = 2ull << 62, kSumMask = kSumOwn - 1ull;
 constexpr int kLookbackTries = 1 << 20;   // polls without progress (about a second) before a block gives up
@@ -321,6 +327,7 @@ struct BuildWs {
     int dup_block;                // ranks per block of the binning and pair emission
     int kpt_depth, kpt_tile;      // keys per thread of the sweeps
     long long nb_depth, nb_tile;  // blocks of a sweep
+    int look_tries;               // polls without progress before a look-back gives up (negative: the first one)
 };
 
 size_t build_ws_layout(int64_t n, int32_t N, int32_t W, int32_t H, int64_t cap, void* base, BuildWs* out);

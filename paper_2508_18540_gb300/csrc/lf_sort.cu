@@ -130,6 +130,7 @@ struct SweepArgs {
     const unsigned long long* n_dev;       // device count (or null)
     int shift;
     int pass;                              // ticket
+    int look_tries;
     const uint32_t* tot;                   // digit totals of this pass
     unsigned long long* stat;              // look-back words [blocks][kDigits]
 };
@@ -160,7 +161,13 @@ __global__ void __launch_bounds__(kSweepThreads, 2) k_sweep(const void* __restri
     SweepSmem<KPT>& S = *reinterpret_cast<SweepSmem<KPT>*>(sweep_raw);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const long long n = a.n_dev ? (long long)*a.n_dev : a.n_static;
-    if (tid == 0) S.tile = atomicAdd(&a.hdr->ticket[a.pass], 1u);
+    if (tid == 0) {
+        // After a wait gave up (in a pass before, or in an earlier block of this
+        // one) no block does anything: the keys may hold stale ones, which the
+        // digit totals don't count, and their places could lie past the arrays.
+        const uint32_t place = atomicAdd(&a.hdr->ticket[a.pass], 1u);
+        S.tile = a.hdr->timeout ? 0xffffffffu : place;   // past any count of keys
+    }
     for (int i = tid; i < kWarps * kDigits; i += kSweepThreads) (&S.wcnt[0][0])[i] = 0u;
     __syncthreads();
     const long long tile = S.tile, blk = tile * (kSweepThreads * KPT);
@@ -249,7 +256,7 @@ __global__ void __launch_bounds__(kSweepThreads, 2) k_sweep(const void* __restri
             }
             t -= u;
             idle = u ? 0 : idle + 1;
-            if (idle > kLookbackTries) {
+            if (idle > a.look_tries) {
                 atomicExch(&a.hdr->timeout, 1);
                 done = true;
             }
@@ -294,10 +301,10 @@ __global__ void __launch_bounds__(256) k_depth_runs(BuildWs w)
     pdl_trigger();
     const long long M = (long long)w.hdr->M;
     const long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= M) return;
+    if (r >= M || w.hdr->timeout) return;   // after a wait gave up valB is not an order
     const uint32_t* key = w.tkeyB;
     auto same = [&](long long i, uint32_t k) { return i >= 0 && i < M && ((key[i] ^ k) & kDepthKeyMask) == 0u; };
-    const uint32_t k = key[r], v = min(w.valB[r], (uint32_t)(w.hdr->n - 1));   // (in bounds after a wait gave up, too)
+    const uint32_t k = key[r], v = w.valB[r];
     const bool left = same(r - 1, k), right = same(r + 1, k);
     if (!left && !right) {
         w.valA[r] = v;
@@ -314,14 +321,14 @@ __global__ void __launch_bounds__(256) k_depth_runs(BuildWs w)
     if (!longer) {
         int before = 0;
         for (long long i = s; i < e; ++i) {
-            const uint32_t u = min(w.valB[i], (uint32_t)(w.hdr->n - 1));
+            const uint32_t u = w.valB[i];
             before += i != r && depth_less(w.keyA[u], u, full, v) ? 1 : 0;
         }
         w.valA[s + before] = v;
         return;
     }
     w.valA[r] = v;
-    if (!left || w.keyA[min(w.valB[r - 1], (uint32_t)(w.hdr->n - 1))] <= full) return;
+    if (!left || w.keyA[w.valB[r - 1]] <= full) return;
     for (s = r; same(s - 1, k);) --s;
     if (atomicOr(&w.tkeyB[s], 0x80000000u) & 0x80000000u) return;   // listed
     while (same(e, k)) ++e;
@@ -442,6 +449,7 @@ void sort_depth_keys(const BuildWs& ws, long long n, cudaStream_t s)
         a.n_dev = pass == 0 ? nullptr : &ws.hdr->M;
         a.shift = pass * kBits;
         a.pass = pass;
+        a.look_tries = ws.look_tries;
         a.tot = ws.dhist + pass * kDigits;
         a.stat = ws.sstat + (size_t)pass * ws.nb_depth * kDigits;
         const int in = (pass + 1) & 1, out = pass & 1;
@@ -470,6 +478,7 @@ void sort_tile_keys(const BuildWs& ws, long long cap, int tile_bits, cudaStream_
         a.n_dev = &ws.hdr->tile_n;
         a.shift = pass * kBits;
         a.pass = kDepthPasses + pass;
+        a.look_tries = ws.look_tries;
         a.tot = ws.dhist + (kDepthPasses + pass) * kDigits;
         a.stat = ws.sstat + ((size_t)kDepthPasses * ws.nb_depth + (size_t)pass * ws.nb_tile) * kDigits;
         sweep<false>(ws.kpt_tile, kb[cur], vb[cur], kb[cur ^ 1], vb[cur ^ 1], a, ws.nb_tile, s);
