@@ -69,6 +69,7 @@ constexpr int kEmitStage = 4096;   // pairs
 // atomic per pair on four words serialises (with the staging above: 48 -> 25 us
 // for 5M pairs on 1024 super-tiles; with fewer pairs the folding costs more).
 constexpr int kFoldSupers = 1024;
+constexpr uint32_t kNoBlock = 0xffffffffu;   // no place among the blocks: a wait gave up
 
 // Chunks and copies (BIN) and pairs (EMIT) of PER ranks per thread, kT apart.
 // One kernel does both for few primitives, where launches and latencies
@@ -95,10 +96,14 @@ __global__ void __launch_bounds__(kT, EMIT ? 4 : 6) k_bin_emit(BuildWs w, BinPar
     __shared__ DispRange s_dr;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const long long M = (long long)w.hdr->M;
-    const uint32_t last_prim = (uint32_t)(w.hdr->n - 1);
     if (tid == 0) {
-        s_block = !EMIT ? blockIdx.x : atomicAdd(&w.hdr->ticket[kDepthPasses + kTilePassesMax], 1u);
-        if (BIN && p.binning != LF_BIN_QUANTILE && M > 0) {
+        // After a wait gave up (of the sort, or in an earlier block here) valA is
+        // no order: no block does anything. (Depths out of order give bins below
+        // zero, and chunk_start would be written there.)
+        const uint32_t place = !EMIT ? blockIdx.x : atomicAdd(&w.hdr->ticket[kDepthPasses + kTilePassesMax], 1u);
+        const bool valid = !w.hdr->timeout;
+        s_block = valid ? place : kNoBlock;
+        if (BIN && valid && p.binning != LF_BIN_QUANTILE && M > 0) {
             DispRange d;
             d.izmin = __ddiv_rn(1.0, rank_depth(w, 0));
             d.span = __dsub_rn(d.izmin, __ddiv_rn(1.0, rank_depth(w, M - 1)));
@@ -116,6 +121,7 @@ __global__ void __launch_bounds__(kT, EMIT ? 4 : 6) k_bin_emit(BuildWs w, BinPar
     }
     __syncthreads();
     const long long b = s_block, r0 = b * (PER * kT);
+    if (s_block == kNoBlock) return;
     if (M == 0) {
         if (BIN && b == 0)
             for (int k = tid; k <= p.N; k += kT) w.chunk_start[k] = 0;
@@ -136,7 +142,7 @@ __global__ void __launch_bounds__(kT, EMIT ? 4 : 6) k_bin_emit(BuildWs w, BinPar
 #pragma unroll
         for (int j = 0; j < PER; ++j) {
             const long long r = r0 + j * kT + tid;
-            g[j] = r < M ? min(w.valA[r], last_prim) : 0u;
+            g[j] = r < M ? w.valA[r] : 0u;
             rc[j] = r < M ? rect[g[j]] : make_int4(0, 0, -1, -1);
         }
 #pragma unroll

@@ -7,8 +7,7 @@ namespace lf {
 
 __device__ __forceinline__ double rank_depth(const BuildWs& w, long long r)
 {
-    // (in bounds after a wait of the sort gave up, too)
-    return __longlong_as_double((long long)w.keyA[min(w.valA[r], (uint32_t)(w.hdr->n - 1))]);
+    return __longlong_as_double((long long)w.keyA[w.valA[r]]);
 }
 
 // member count and distance of plane k

@@ -36,7 +36,7 @@ CASES = [("sort", 10000, 0.01, 200), ("sort", 200000, 0.003, 200), ("bin", 1500,
 
 
 @pytest.mark.parametrize("first,n,radius,size", CASES)
-@pytest.mark.parametrize("binning", ["quantile"])
+@pytest.mark.parametrize("binning", ["quantile", "disparity"])
 def test_build_waits_that_give_up(first, n, radius, size, binning):
     args = (S.identity_camera(size, 50.0), S.display_for(3.0, 0.1), S.ViewSet(3), 16, binning, "f32")
     g = api.DeviceGaussians.from_scene(_scene(n, radius))
