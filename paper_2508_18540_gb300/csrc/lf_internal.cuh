@@ -281,6 +281,11 @@ struct WsHeader {
     int timeout;                  // a bounded wait of the build gave up
 };
 
+// The build made no lists, and its order may be none: the adjoints give zero gradients.
+#ifdef __CUDACC__
+__device__ __forceinline__ bool no_lists(const WsHeader& h) { return h.overflow || h.timeout; }
+#endif
+
 // Split lists of the Gaussian raster: a list of L > r_seg entries is cut into
 // ceil(L / r_seg) parts, each with a partial (C, T) slot of one super-tile
 // (kSuper^2 texels); r_seg is at least kRasterSegMin and large enough that

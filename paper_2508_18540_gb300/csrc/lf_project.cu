@@ -343,7 +343,7 @@ __global__ void __launch_bounds__(kProjThreads) k_project_voxels(lf_voxels v, Pr
 __global__ void __launch_bounds__(256) k_gauss_chain(lf_gaussians g, ProjParams p, BuildWs w, lf_gaussians_grad out)
 {
     const long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (w.hdr->overflow || r >= (long long)w.hdr->M) return;
+    if (no_lists(*w.hdr) || r >= (long long)w.hdr->M) return;
     const uint32_t i = w.valA[r];
     const float4 a0 = reinterpret_cast<const float4*>(w.g2d)[3 * r];
     const float4 a1 = reinterpret_cast<const float4*>(w.g2d)[3 * r + 1];
@@ -464,7 +464,7 @@ __global__ void __launch_bounds__(256) k_gauss_chain(lf_gaussians g, ProjParams 
 __global__ void __launch_bounds__(256) k_voxel_scatter(BuildWs w, lf_voxels_grad out)
 {
     const long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (w.hdr->overflow || r >= (long long)w.hdr->M) return;
+    if (no_lists(*w.hdr) || r >= (long long)w.hdr->M) return;
     const uint32_t i = w.valA[r];
     const float4* a = reinterpret_cast<const float4*>(w.g2d) + 3 * r;
     const float4 a0 = a[0], a1 = a[1], a2 = a[2];

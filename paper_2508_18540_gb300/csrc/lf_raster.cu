@@ -963,7 +963,7 @@ __global__ void __launch_bounds__(kGaussBwdThreads, 3) k_raster_gauss_bwd(BuildW
                                                                       float4* __restrict__ g2d)
 {
     __shared__ GaussBwdSmem sm;
-    if (w.hdr->overflow) return;
+    if (no_lists(*w.hdr)) return;
     const long long b = blockIdx.x;
     if (b < w.r_nslots) {
         if (b >= (long long)w.hdr->r_heavy) return;
@@ -1085,7 +1085,7 @@ __global__ void __launch_bounds__(kTilePix) k_raster_voxel_bwd(BuildWs w, Raster
     constexpr int NT = kTilePix;
     extern __shared__ __align__(16) unsigned char vox_smem[];
     VoxBwdSmem& sm = *reinterpret_cast<VoxBwdSmem*>(vox_smem);
-    if (w.hdr->overflow) return;
+    if (no_lists(*w.hdr)) return;
     const int t = blockIdx.x, k = blockIdx.y;
     const int tx = t % p.tiles_x, ty = t / p.tiles_x;
     const int lx = threadIdx.x & (kTile - 1), ly = threadIdx.x / kTile;

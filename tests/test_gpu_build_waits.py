@@ -57,6 +57,20 @@ def test_build_waits_that_give_up(first, n, radius, size, binning):
     assert b"gave up" in L.load().lf_last_error()
     for t in (r.planes.rgba, r.planes.d, r.planes.count):
         assert not t.any()
+    # the adjoint of the empty planes: no gradient, whatever the lost places hold
+    # (the voxels' adjoint reads the same header and order)
+    dplanes = torch.ones((r.N, r.ref.H, r.ref.W, 4), dtype=torch.float32, device="cuda")
+    v = api.DeviceVoxels.from_scene(S.VoxelScene(np.zeros((n, 3), np.int32), np.zeros(n, np.uint8), np.zeros(3), 1.0,
+                                                 np.ones((n, 8), np.float32), np.ones((n, 3), np.float32)))
+    gg, gv = api.GaussianGrads.empty(n, "cuda"), api.VoxelGrads.empty(n, "cuda")
+    fields = list(vars(gg).values()) + list(vars(gv).values())
+    for t in fields:
+        t.fill_(3)
+    api.lf_build_mpi_backward_gaussians(g, r.ref, r.planes, dplanes, gg, r.ws)
+    api.lf_build_mpi_backward_voxels(v, r.ref, r.planes, dplanes, gv, r.ws)
+    torch.cuda.synchronize()
+    for t in fields:
+        assert not t.any()
     again = r.build(g)
     assert r.status() == (L.LF_OK, pairs, M)
     for a, b in zip((again.rgba, again.d, again.count, again.chunk, again.rect),
