@@ -76,3 +76,19 @@ def test_build_waits_that_give_up(first, n, radius, size, binning):
     for a, b in zip((again.rgba, again.d, again.count, again.chunk, again.rect),
                     (want.rgba, want.d, want.count, want.chunk, want.rect)):
         assert torch.equal(a, b)
+
+
+def test_batch_status_after_a_build_that_gave_up():
+    wls = [S.workload_display(seed=30 + i, n=n, res=64, N=8, V=5) for i, n in enumerate((5000, 3000))]
+    b = api.BatchRenderer(wls, "f32")
+    b.render()
+    assert b.status() == L.LF_OK
+    want = [o.clone() for o in b.outputs]
+    r, g, planes = b.parts[1]
+    api.lf_selftest_build_waits(g, r.ref, r.N, wls[1].binning, r.ws, planes, b.stream)
+    assert b.status() == L.LF_ERR_TIMEOUT
+    b.render()
+    assert b.status() == L.LF_OK
+    for o, w in zip(b.outputs, want):
+        assert torch.equal(o, w)
+    b.close()
