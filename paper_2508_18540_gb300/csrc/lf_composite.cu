@@ -159,8 +159,6 @@ __global__ void k_wait_selftest(unsigned long long limit_ns, int* result)
     *result = mbar_wait_for(b, 0u, limit_ns) ? 2 : 1;
 }
 
-constexpr size_t kCompSmemMax = 200 * 1024;
-
 // Texels that a group of VG views spreads over on the planes from a quarter
 // of the focal distance (from the reference camera) on.
 double view_spread(const CompParams& p, int VG)
@@ -220,7 +218,7 @@ void launch_fwd(const CompParams& p, const CompGeom& G, const void* planes, cons
                 cudaStream_t s)
 {
     auto kern = k_composite_staged<DT, BILINEAR, VG, SAVE>;
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G.smem_bytes);
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCompSmemMax);
     const dim3 grid((unsigned)(G.groups_x * p.Vy * ((p.Nx + G.TX - 1) / G.TX)), (unsigned)((p.Ny + G.BY - 1) / G.BY));
     launch_pdl(kern, grid, dim3(kCompBlock), G.smem_bytes, s, p, G, static_cast<const char*>(planes), ws, out, state);
 }

@@ -930,6 +930,11 @@ __device__ __forceinline__ void composite_tile(const CompParams& p, const CompGe
     }
 }
 
+// Most dynamic shared memory of a layout. Every launch sets its kernel's limit
+// to this, whatever it needs: the limit is the kernel's, and one set to a
+// launch's own size would refuse a larger launch of another thread.
+constexpr size_t kCompSmemMax = 200 * 1024;
+
 // CTAs per SM that the adjoint's registers leave room for
 __host__ __device__ constexpr int comp_bwd_ctas(int VG) { return VG > 3 ? 4 : 6; }
 

@@ -38,7 +38,7 @@ template <int DT, bool BILINEAR, int VG>
 void launch_batched(const CompScene* scs, int n_sc, long long total, size_t smem, cudaStream_t s)
 {
     auto kern = k_composite_batched<DT, BILINEAR, VG>;
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCompSmemMax);
     kern<<<(unsigned)total, kCompBlock, smem, s>>>(scs, n_sc);
 }
 

@@ -446,7 +446,7 @@ void launch_bwd(const CompParams& p, const CompGeom& G, const void* planes, cons
                 float4* dplanes, const float4* state, cudaStream_t s)
 {
     auto kern = k_composite_bwd_staged<DT, BILINEAR, VG, FS>;
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G.smem_bytes);
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCompSmemMax);
     const dim3 grid((unsigned)(G.groups_x * p.Vy * ((p.Nx + G.TX - 1) / G.TX)), (unsigned)((p.Ny + G.BY - 1) / G.BY));
     launch_pdl(kern, grid, dim3(kCompBlock), G.smem_bytes, s, p, G, static_cast<const char*>(planes), ws, dviews, dplanes,
                state);

@@ -310,14 +310,19 @@ __global__ void __launch_bounds__(kFusedThreads, 4) k_filter_fused(void* planes,
     }
 }
 
+constexpr int fused_pitch(int radius) { return (kStrip + 2 * radius + 31) / 32 * 32; }
+
 template <int DT>
 void launch_fused(void* planes, int N, int W, int H, const FilterParams& f, cudaStream_t s)
 {
     const int strips = (W + kStrip - 1) / kStrip;
-    const int pitch = (kStrip + 2 * f.radius + 31) / 32 * 32, ring = kBand + 2 * f.radius <= 32 ? 32 : 64;
+    const int pitch = fused_pitch(f.radius), ring = kBand + 2 * f.radius <= 32 ? 32 : 64;
     const size_t smem = sizeof(float4) * (size_t)(kBand * pitch + ring * kStrip);
     auto kern = k_filter_fused<DT>;
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // (the limit of the widest filter: one set to this launch's own size would
+    // refuse a wider filter that another thread launches at the same time)
+    constexpr size_t smem_max = sizeof(float4) * (size_t)(kBand * fused_pitch(kFilterMaxRadius) + 64 * kStrip);
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)strips, (unsigned)N);
     cfg.blockDim = dim3(kFusedThreads);
