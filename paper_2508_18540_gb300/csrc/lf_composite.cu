@@ -159,12 +159,13 @@ __global__ void k_wait_selftest(unsigned long long limit_ns, int* result)
     *result = mbar_wait_for(b, 0u, limit_ns) ? 2 : 1;
 }
 
-// Texels that a group of VG views spreads over on the planes from a quarter
-// of the focal distance (from the reference camera) on.
-double view_spread(const CompParams& p, int VG)
+// Texels that a group of VG views spreads over on the planes from nearest times
+// the focal distance (from the reference camera) on.
+constexpr double kNearest = 0.25;
+double view_spread(const CompParams& p, int VG, double nearest = kNearest)
 {
     if (p.Vx < 2) return 0.0;
-    const double near = 0.25 * p.D_focal, views = (VG < p.Vx ? VG : p.Vx) - 1;
+    const double near = nearest * p.D_focal, views = (VG < p.Vx ? VG : p.Vx) - 1;
     const double near_shift = std::fabs(p.D_focal - p.D_forward - near) / (near * p.tthp_x), far_shift = 1.0 / p.tthp_x;
     return 0.5 * p.W * views * 2.0 * p.tphi_x / (p.Vx - 1) * (near_shift > far_shift ? near_shift : far_shift);
 }
@@ -180,7 +181,7 @@ int tile_columns(const CompParams& p, int VG, int most)
     double best_cost = 1e300;
     for (int tx : {128, 64, 32}) {
         if (tx > most) continue;
-        const double window = tx * kAdvance * p.P_s + view_spread(p, VG);
+        const double window = tx * kAdvance * p.P_s + view_spread(p, VG, p.bilinear ? 0.5 : kNearest);
         const double cost = (double)((p.Nx + tx - 1) / tx * tx) * (tx == 128 ? 1.0 : tx == 64 ? 1.02 : 1.05) *
                             (1.0 + 0.4 * (p.bilinear ? 2.0 : 1.0) * window / ((double)tx * VG));
         if (cost < best_cost) best_cost = cost, best = tx;
@@ -190,15 +191,18 @@ int tile_columns(const CompParams& p, int VG, int most)
 
 constexpr double kSMs = 152.0;
 
-// Views per thread: the least waves of CTAs times (VG + 3) per CTA and CTAs
+// Views per thread: the least waves of CTAs times (VG + fixed) per CTA and CTAs
 // per SM. The fixed cost of a view group (staging every plane's window) is
 // worth about three views. A last, partly filled wave counts half a wave and
 // half of what fills it (its CTAs have the SM to fewer): it decides where the
 // grid is small -- 9 views of 128^2, N 16: 3 views per thread run 2 % faster
 // than 9 (0.142 against 0.146 ms a frame); 9 of 256^2 bilinear: 9 run 7 %
 // faster than 3; 45 of 512^2: 15 run 6 % faster than 9.
+// The bilinear adjoint's cost goes almost by the sample, a group's fixed cost
+// is about 0.6 views: 45 views of 256^2, 9 per thread 2.29 ms a fitting step, 3
+// per thread 2.49; 12 views 1.26 and 0.95.
 template <typename Ctas>
-int views_per_thread(const CompParams& p, std::initializer_list<int> options, Ctas ctas)
+int views_per_thread(const CompParams& p, std::initializer_list<int> options, double fixed, Ctas ctas)
 {
     int best = 1;
     double best_cost = 1e300;
@@ -207,7 +211,7 @@ int views_per_thread(const CompParams& p, std::initializer_list<int> options, Ct
         const double tiles = (double)((p.Nx + tx - 1) / tx) * ((p.Ny + by - 1) / by) * p.Vy;
         const double waves = tiles * ((p.Vx + vg - 1) / vg) / (kSMs * ctas(vg)), whole = std::floor(waves);
         const double part = waves - whole;
-        const double cost = (whole + (part > 0.0 ? 0.5 + 0.5 * part : 0.0)) * (vg + 3) * ctas(vg);
+        const double cost = (whole + (part > 0.0 ? 0.5 + 0.5 * part : 0.0)) * (vg + fixed) * ctas(vg);
         if (cost < best_cost) best_cost = cost, best = vg;
     }
     return best;
@@ -256,12 +260,13 @@ struct FwdLaunch {
 
 int comp_views_fwd(const CompParams& p)
 {
-    return views_per_thread(p, {15, 9, 5, 3, 1}, [&](int vg) { return comp_ctas(vg, p.bilinear != 0, p.dtype); });
+    return views_per_thread(p, {15, 9, 5, 3, 1}, 3.0, [&](int vg) { return comp_ctas(vg, p.bilinear != 0, p.dtype); });
 }
 
 int comp_views_bwd(const CompParams& p)
 {
-    return views_per_thread(p, {9, 3}, [](int vg) { return comp_bwd_ctas(vg); });
+    const bool bilinear = p.bilinear != 0;
+    return views_per_thread(p, {9, 3}, bilinear ? 0.6 : 3.0, [&](int vg) { return comp_bwd_ctas(vg, bilinear); });
 }
 
 // Staged layout of one composite (see CompGeom). The stage holds the window
@@ -280,20 +285,32 @@ CompGeom comp_geom(const CompParams& p, const void* planes, int VG, bool save, b
     G.groups_x = (p.Vx + VG - 1) / VG;
     G.bulk = ((uintptr_t)planes) % 16 == 0 && ((size_t)p.W * TB) % 16 == 0;
     G.hdr_bytes = (uint32_t)(VG == 1 ? 0 : 16 * ((VG + 3) / 4));
-    const double spread = view_spread(p, VG), advance = kAdvance * p.P_s;
-    // per-warp rows, bilinear: the blended row; the adjoint's gradient sums
-    const double warp_tex = 32.0 * advance + spread + 4.0;
-    G.wcap = (uint32_t)(warp_tex < 512.0 ? warp_tex : 512.0) / 8 * 8;
-    const size_t rows = p.bilinear ? (size_t)kWarps * G.wcap * 16 * (bwd ? 3 : 1) : 0;
+    const double advance = kAdvance * p.P_s;
     const size_t stop = save ? 4 * (size_t)kCompThreads * VG : 0;
     const size_t ctrl = 16 * kStages + 16 + 16 * kDescs + (size_t)kDescs * (p.bilinear ? 64 : kDescBytes);
-    const size_t fixed = rows + ctrl + stop + 128;
-    const int ctas = bwd ? comp_bwd_ctas(VG) : comp_ctas(VG, p.bilinear != 0, p.dtype);
+    const int ctas = bwd ? comp_bwd_ctas(VG, p.bilinear != 0) : comp_ctas(VG, p.bilinear != 0, p.dtype);
     const size_t budget = (size_t)(227 * 1024) / ctas - 1024;
     const size_t full = round16((size_t)p.W * TB) + 16;   // and the zero texel
-    const double tile_tex = G.TX * advance + spread + 4.0 + 48.0 / (double)TB;
-    const size_t need = tile_tex * (double)TB < (double)full ? round16((size_t)tile_tex * TB) : full;
     auto stage = [&](size_t win) { return kPair * (G.hdr_bytes + win * G.BY * rpy); };
+    size_t rows = 0, fixed = 0, need = 0;
+    // Bilinear, few views far apart: the windows of near planes alone can take
+    // so much shared memory that fewer CTAs run than the registers allow, with
+    // two stages each (FP32, 3 x 2 views of 323^2, N 69, a fitting step: 1.19 ms
+    // with windows from a quarter of the focal distance on, 1.08 from 0.35 on;
+    // 3 views of 512^2: 185 and 162 us from half of it on). Then only planes
+    // further away get windows, up to half the focal distance: a display
+    // focused at the middle disparity of its scene has no nearer ones.
+    for (double nearest : {kNearest, 0.35, 0.5}) {
+        const double spread = view_spread(p, VG, nearest);
+        // per-warp rows, bilinear: the blended row; the adjoint's gradient sums
+        const double warp_tex = 32.0 * advance + spread + 4.0;
+        G.wcap = (uint32_t)(warp_tex < 512.0 ? warp_tex : 512.0) / 8 * 8;
+        rows = p.bilinear ? (size_t)kWarps * G.wcap * 16 * (bwd ? 3 : 1) : 0;
+        fixed = rows + ctrl + stop + 128;
+        const double tile_tex = G.TX * advance + spread + 4.0 + 48.0 / (double)TB;
+        need = tile_tex * (double)TB < (double)full ? round16((size_t)tile_tex * TB) : full;
+        if (!p.bilinear || fixed + 3 * stage(need) <= budget) break;
+    }
     G.stages = kStages;
     while (G.stages > 2 && fixed + G.stages * stage(need) > budget) --G.stages;
     while (G.stages > 2 && fixed + G.stages * stage(need) > kCompSmemMax) --G.stages;

@@ -864,9 +864,11 @@ __device__ __forceinline__ void composite_tile(const CompParams& p, const CompGe
                 const RowPair rp(p, tg, B.x, B.y);
                 const int lo = (int)lds_u32(d + 32 + 4 * (tid >> 5)), n = (int)lds_u32(d + 48 + 4 * (tid >> 5));
                 // blending a warp's window first pays while it is read more often than it is
-                // made: 3 accesses per 32 texels against 2 saved per view (few views that
-                // lie far apart have wide windows)
-                const bool direct = VG <= 5 && mode != kGlobal && 3 * ((n + 31) / 32) > 2 * VG;
+                // made, some 2 accesses per 32 texels against one saved per view (few views
+                // that lie far apart have wide windows): 3 views of 512^2, N 64, FP32 162 us
+                // with a line at 2/3, 152 at 1/2; RGBA8 texels, which need unpacking, 197 and 262
+                const bool direct = VG <= 5 && mode != kGlobal &&
+                                    (DT == LF_U8 ? 3 * ((n + 31) / 32) > 2 * VG : 2 * ((n + 31) / 32) > VG);
                 if (n > 0 && direct) {
                     const uint32_t r0 = sa + tg.row, c = (uint32_t)(tg.pxm - __float_as_int(A.y));
                     ViewH vh;
@@ -935,16 +937,25 @@ __device__ __forceinline__ void composite_tile(const CompParams& p, const CompGe
 // launch's own size would refuse a larger launch of another thread.
 constexpr size_t kCompSmemMax = 200 * 1024;
 
-// CTAs per SM that the adjoint's registers leave room for
-__host__ __device__ constexpr int comp_bwd_ctas(int VG) { return VG > 3 ? 4 : 6; }
+// CTAs per SM that the adjoint's registers leave room for: nearest, bound by
+// its atomics, 9 views at 96 registers, 3 at 64; bilinear 9 at 128 and 3 at 96,
+// without spills (fitting steps of 256^2, N 64, 12 views: 1.32 ms with 96 and
+// 64, 0.95 now; 45 views 2.72 and 2.29).
+__host__ __device__ constexpr int comp_bwd_ctas(int VG, bool bilinear)
+{
+    return bilinear ? (VG > 3 ? 3 : 4) : (VG > 3 ? 4 : 6);
+}
 
 // CTAs per SM of the forward, that is, registers per thread: nearest 15 views
 // at 96, 9 at 72 (FP32 planes; the others, whose texels take fewer registers,
 // at 64), bilinear 15 at 128 (three CTAs: 0.91 ms on FP16 planes, 45 views of
-// 512^2, N 64; at 96 registers spills take it to 1.03).
+// 512^2, N 64; at 96 registers spills take it to 1.03), fewer at 96 (FP32, 5
+// views of 256^2, N 64: 92 us at six CTAs and 64 registers, with spills, 65
+// now; 2 views 72 and 52), but RGBA8, 3 views and fewer, which has the shortest
+// windows, at five CTAs (2 x 2 views of 400^2, N 50: 214 us at four, 197 now).
 __host__ __device__ constexpr int comp_ctas(int VG, bool bilinear, int dtype)
 {
-    return bilinear ? (VG > 9 ? 3 : VG > 5 ? 4 : 6) : (VG > 9 ? 4 : VG > 5 ? (dtype == LF_F32 ? 5 : 6) : 7);
+    return bilinear ? (VG > 9 ? 3 : VG > 3 || dtype != LF_U8 ? 4 : 5) : (VG > 9 ? 4 : VG > 5 ? (dtype == LF_F32 ? 5 : 6) : 7);
 }
 
 // f.template operator()<DT, BILINEAR>() for the run-time plane type and sampling

@@ -109,7 +109,7 @@ __device__ __forceinline__ bool step_back(BwdViews<VG>& s, int jj, int k, float4
 // FS: started from the state the saving forward wrote (one walk, back to
 // front); else a front-to-back walk of the opacities first.
 template <int DT, bool BILINEAR, int VG, bool FS>
-__global__ void __launch_bounds__(kCompBlock, comp_bwd_ctas(VG))
+__global__ void __launch_bounds__(kCompBlock, comp_bwd_ctas(VG, BILINEAR))
     k_composite_bwd_staged(const __grid_constant__ CompParams p, const __grid_constant__ CompGeom G,
                            const char* __restrict__ planes, const __grid_constant__ CompWs w,
                            const float4* __restrict__ dviews, float4* __restrict__ dplanes,
