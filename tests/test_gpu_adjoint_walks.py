@@ -1,0 +1,48 @@
+"""The composite adjoint where its walks end early: opaque texels, more planes
+than descriptors in shared memory, views past one group, ragged rows. References
+and tolerances are those of test_gpu_staged_composite (FP64 autograd)."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2508_18540_gb300 import api
+from paper_2508_18540_gb300 import synth as S
+from tests.test_gpu_staged_composite import _adjoint64, _built, _case, orc  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+
+
+# opaque: the share of opaque 4 x 4 blocks in every plane, or the plane from
+# which on every texel is opaque; planes in all (90: of these 72 not empty)
+@pytest.mark.parametrize("bilinear", [False, True])
+@pytest.mark.parametrize("dtype,Nx,Vx,N,opaque", [
+    ("f32", 64, 4, 12, 0.5), ("f16", 64, 4, 12, 0.9), ("f16", 67, 4, 12, 0.5), ("u8", 67, 4, 12, 0.9),
+    ("f32", 40, 12, 90, 0.02), ("bf16", 41, 12, 90, 0.02), ("f32", 130, 5, 14, 3), ("u8", 33, 11, 90, 70)])
+def test_opaque_texels_against_autograd(orc, dtype, Nx, Vx, N, opaque, bilinear):  # noqa: F811
+    views = S.ViewSet(Vx, 1, bilinear, (0.1, 0.2, 0.3))
+    Ny = 4
+    cam, disp, ref, pl, vals, d, count, ws = _case(dtype, 1, Nx, Ny, views, N, seed=5)
+    rng = np.random.default_rng(1)
+    if isinstance(opaque, float):
+        hit = rng.random((N, (Ny + 3) // 4, (Nx + 3) // 4)) < opaque
+        hit = np.repeat(np.repeat(hit, 4, 1), 4, 2)[:, :Ny, :Nx]
+    else:
+        hit = np.zeros(vals.shape[:3], bool)
+        hit[opaque:] = True
+    pl.rgba[..., 3][torch.from_numpy(hit).cuda()] = 255 if dtype == "u8" else 1.0
+    vals[..., 3][hit] = 1.0
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    dv = torch.randn((Vx, Ny, Nx, 4), device="cuda", generator=gen)
+    want = _adjoint64(orc, cam, disp, vals, d, count, views, dv)
+    tol = (1e-3 if bilinear else 2e-5) * np.abs(want).max()
+    got = torch.full(vals.shape, float("nan"), device="cuda")
+    api.lf_composite_backward(pl, ref, views, dv, got, ws)
+    assert api.lf_composite_status(N, views, ws) == 0
+    assert np.abs(got.cpu().numpy() - want).max() <= tol
+    out = torch.empty(api.views_shape(views, Nx, Ny), device="cuda")
+    state = torch.empty(api.composite_state_shape(ref, views), device="cuda")
+    api.lf_composite_save(pl, ref, views, out, state, ws)
+    got.fill_(float("nan"))
+    api.lf_composite_backward_saved(pl, ref, views, dv, state, got, ws)
+    assert api.lf_composite_status(N, views, ws) == 0
+    assert np.abs(got.cpu().numpy() - want).max() <= tol
