@@ -101,11 +101,22 @@ __device__ __forceinline__ float rcp_approx(float x)
 
 // The view's step back over a plane sampled as t: T in front of it, the texel
 // gradient (T g_rgb, -T B), and B in front of it. False: no gradient.
-template <int VG>
+// T / oma is T times the approximate reciprocal; EXACT adds one correction by
+// the quotient's own remainder (Markstein, IBM J. Res. Dev. 34, 1990), within a
+// rounding of the true quotient. FP32 planes go without, as their kernel always
+// did (3 % of a 512^2 adjoint); the others, whose ragged rows were divided, have
+// it (ragged FP16, 21 views of 301^2, N 60: 642 -> 662 us, with the division
+// itself 808).
+template <bool EXACT, int VG>
 __device__ __forceinline__ bool step_back(BwdViews<VG>& s, int jj, int k, float4 t, float4* gt)
 {
     const float oma = 1.0f - t.w;
-    if (k < s.stop[jj] && oma > 0.0f) s.T[jj] *= rcp_approx(oma);
+    if (k < s.stop[jj] && oma > 0.0f) {
+        const float r = rcp_approx(oma);
+        float q = s.T[jj] * r;
+        if (EXACT) q = fmaf(fmaf(-q, oma, s.T[jj]), r, q);
+        s.T[jj] = q;
+    }
     const float T = s.T[jj], B = s.B[jj];
     const float4 g = s.g[jj];
     *gt = make_float4(T * g.x, T * g.y, T * g.z, -T * B);
@@ -125,6 +136,7 @@ __global__ void __launch_bounds__(kCompBlock, comp_bwd_ctas(VG, BILINEAR))
     extern __shared__ __align__(128) unsigned char smem[];
     const TileSmem sm(G, smem);
     constexpr bool LONG = BILINEAR;   // descriptors with the warps' windows
+    constexpr bool kExact = DT != LF_F32;
     __shared__ int s_kmax, s_n;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int nvg = G.groups_x * p.Vy;
@@ -315,7 +327,7 @@ __global__ void __launch_bounds__(kCompBlock, comp_bwd_ctas(VG, BILINEAR))
         s.B[jj] = fmaf(s.g[jj].x, p.bg[0], fmaf(s.g[jj].y, p.bg[1], fmaf(s.g[jj].z, p.bg[2], -s.g[jj].w)));
     }
 
-    // back to front: T by division, texel gradients, the B recurrence
+    // back to front: T, texel gradients, the B recurrence
     for (int i0 = 0; i0 < n2; i0 += kPair, ring.next(G.stages)) {
         if (!mbar_wait_bounded(sm.full + 8 * ring.st, ring.ph)) {
             atomicExch(w.err, 1);
@@ -369,7 +381,7 @@ __global__ void __launch_bounds__(kCompBlock, comp_bwd_ctas(VG, BILINEAR))
 #pragma unroll
                     for (int e = 0; e < 3 && 3 * t + e < VG; ++e) {
                         float4 gt;
-                        if (!step_back(s, 3 * t + e, k, tx[e], &gt) || !in[e]) gt = zero4, b[e] = rb;
+                        if (!step_back<kExact>(s, 3 * t + e, k, tx[e], &gt) || !in[e]) gt = zero4, b[e] = rb;
                         const bool fresh = b[e] != rb;
                         if (fresh && rb) atomicAdd(drow + rb, run);
                         run.x = fresh ? gt.x : run.x + gt.x;
@@ -410,7 +422,7 @@ __global__ void __launch_bounds__(kCompBlock, comp_bwd_ctas(VG, BILINEAR))
                         u0 = sample_global<DT>(p, planes, k, rp, i0, &u1);
                     }
                     float4 gt;
-                    const bool add = step_back(s, jj, k, mix_taps(wx, u0, u1), &gt);
+                    const bool add = step_back<kExact>(s, jj, k, mix_taps(wx, u0, u1), &gt);
                     if (sums) {
                         if (add && c0) add_smem(acc + o0, make_float4(wa * gt.x, wa * gt.y, wa * gt.z, wa * gt.w));
                         __syncwarp();
