@@ -174,15 +174,21 @@ constexpr double kAdvance = 1.3;   // most texels (over P_s) between neighbourin
 
 // Columns of a tile, at most `most`: 128, 64 or 32, whichever pads and stages
 // least: a narrower tile pads the view's width less and stages relatively
-// wider windows (a staged texel costs about 0.4 of a sample).
-int tile_columns(const CompParams& p, int VG, int most)
+// wider windows (a staged texel costs about 0.4 of a sample). Ragged rows are
+// copied texel by texel, row after row, by the producer warp, which a tile of
+// several rows of the forward waits for (the adjoint has more to do): with 128, 64 and 32 columns, 10 views of 251^2, N 150,
+// FP16, take 93, 107 and 144 us, 16 views of 151 x 110, N 128, BF16, 94, 82 and
+// 108, 16 views of 203 x 150, N 128, BF16, 105, 114 and 127.
+int tile_columns(const CompParams& p, int VG, int most, bool bwd)
 {
+    const bool ragged = !bwd && (size_t)p.W * texel_bytes(p.dtype) % 16 != 0;
+    const double by_64 = ragged ? 1.1 : 1.02, by_32 = ragged ? 1.5 : 1.05;
     int best = 32;
     double best_cost = 1e300;
     for (int tx : {128, 64, 32}) {
         if (tx > most) continue;
         const double window = tx * kAdvance * p.P_s + view_spread(p, VG, p.bilinear ? 0.5 : kNearest);
-        const double cost = (double)((p.Nx + tx - 1) / tx * tx) * (tx == 128 ? 1.0 : tx == 64 ? 1.02 : 1.05) *
+        const double cost = (double)((p.Nx + tx - 1) / tx * tx) * (tx == 128 ? 1.0 : tx == 64 ? by_64 : by_32) *
                             (1.0 + 0.4 * (p.bilinear ? 2.0 : 1.0) * window / ((double)tx * VG));
         if (cost < best_cost) best_cost = cost, best = tx;
     }
@@ -202,12 +208,12 @@ constexpr double kSMs = 152.0;
 // is about 0.6 views: 45 views of 256^2, 9 per thread 2.29 ms a fitting step, 3
 // per thread 2.49; 12 views 1.26 and 0.95.
 template <typename Ctas>
-int views_per_thread(const CompParams& p, std::initializer_list<int> options, double fixed, Ctas ctas)
+int views_per_thread(const CompParams& p, std::initializer_list<int> options, bool bwd, double fixed, Ctas ctas)
 {
     int best = 1;
     double best_cost = 1e300;
     for (int vg : options) {
-        const int tx = tile_columns(p, vg, 128), by = kCompThreads / tx;
+        const int tx = tile_columns(p, vg, 128, bwd), by = kCompThreads / tx;
         const double tiles = (double)((p.Nx + tx - 1) / tx) * ((p.Ny + by - 1) / by) * p.Vy;
         const double waves = tiles * ((p.Vx + vg - 1) / vg) / (kSMs * ctas(vg)), whole = std::floor(waves);
         const double part = waves - whole;
@@ -260,13 +266,13 @@ struct FwdLaunch {
 
 int comp_views_fwd(const CompParams& p)
 {
-    return views_per_thread(p, {15, 9, 5, 3, 1}, 3.0, [&](int vg) { return comp_ctas(vg, p.bilinear != 0, p.dtype); });
+    return views_per_thread(p, {15, 9, 5, 3, 1}, false, 3.0, [&](int vg) { return comp_ctas(vg, p.bilinear != 0, p.dtype); });
 }
 
 int comp_views_bwd(const CompParams& p)
 {
     const bool bilinear = p.bilinear != 0;
-    return views_per_thread(p, {9, 3}, bilinear ? 0.6 : 3.0, [&](int vg) { return comp_bwd_ctas(vg, bilinear); });
+    return views_per_thread(p, {9, 3}, true, bilinear ? 0.6 : 3.0, [&](int vg) { return comp_bwd_ctas(vg, bilinear); });
 }
 
 // Staged layout of one composite (see CompGeom). The stage holds the window
@@ -279,7 +285,7 @@ CompGeom comp_geom(const CompParams& p, const void* planes, int VG, bool save, b
     std::memset(&G, 0, sizeof(G));
     const size_t TB = (size_t)texel_bytes(p.dtype);
     const int rpy = p.bilinear ? 2 : 1;
-    G.TX = tile_columns(p, VG, tile_x);
+    G.TX = tile_columns(p, VG, tile_x, bwd);
     G.BY = kCompThreads / G.TX;
     G.VG = VG;
     G.groups_x = (p.Vx + VG - 1) / VG;
