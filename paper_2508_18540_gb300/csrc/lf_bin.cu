@@ -101,12 +101,14 @@ __global__ void __launch_bounds__(kT, EMIT ? 4 : 6) k_bin_emit(BuildWs w, BinPar
         // no order: no block does anything. (Depths out of order give bins below
         // zero, and chunk_start would be written there.)
         const uint32_t place = !EMIT ? blockIdx.x : atomicAdd(&w.hdr->ticket[kDepthPasses + kTilePassesMax], 1u);
+        const bool disparity = BIN && p.binning != LF_BIN_QUANTILE && M > 0;
+        const uint32_t first = disparity ? w.valA[0] : 0u, last = disparity ? w.valA[M - 1] : 0u;   // beside the flag's load
         const bool valid = !w.hdr->timeout;
         s_block = valid ? place : kNoBlock;
-        if (BIN && valid && p.binning != LF_BIN_QUANTILE && M > 0) {
+        if (disparity && valid) {
             DispRange d;
-            d.izmin = __ddiv_rn(1.0, rank_depth(w, 0));
-            d.span = __dsub_rn(d.izmin, __ddiv_rn(1.0, rank_depth(w, M - 1)));
+            d.izmin = __ddiv_rn(1.0, __longlong_as_double((long long)w.keyA[first]));
+            d.span = __dsub_rn(d.izmin, __ddiv_rn(1.0, __longlong_as_double((long long)w.keyA[last])));
             d.izminf = __double2float_rn(d.izmin);
             d.scale = (float)p.N / __double2float_rn(d.span);
             d.margin = 4.76837158e-7f * (d.scale * d.izminf + 2.0f * (float)p.N);   // 2^-21
