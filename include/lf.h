@@ -353,9 +353,10 @@ lf_status lf_composite_save(const lf_planes* planes, const lf_ref_camera* ref, c
 /* lf_composite_backward from the state lf_composite_save wrote for the same
  * planes, ref and views: one back-to-front walk over the planes instead of
  * two. The planes behind a pixel's stop plane get no gradient from it (their
- * T, below 2^-24, is taken as 0), and the alpha gradient of a stop plane k
- * with T_k below 2^-18 leaves their colours out; otherwise the same gradients
- * up to FP32 rounding. Same contract and errors as lf_composite_backward, and
+ * T, below 2^-24, is taken as 0), and the alpha gradient of a stop plane may
+ * leave their colours out: where plane rows start on 16-byte boundaries, or
+ * T_k is below 2^-18 (the two-walk adjoint: where the rows do). Otherwise the
+ * same gradients up to FP32 rounding. Same contract and errors as lf_composite_backward, and
  * LF_ERR_INVALID_ARG for a NULL, misaligned or short state. */
 lf_status lf_composite_backward_saved(const lf_planes* planes, const lf_ref_camera* ref, const lf_view_set* views,
                                       const float* dviews, const float* state, size_t state_bytes, float* dplanes,

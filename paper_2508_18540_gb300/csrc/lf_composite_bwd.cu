@@ -43,15 +43,18 @@ namespace {
 // wider than the warp's, add straight to dplanes.
 // The planes behind the last stop plane of a warp's pixels in a triple of
 // views (view columns 3 m .. 3 m + 2) are not walked for it: they carry T = 0
-// for all of them, and what the stop planes' alpha gradients miss is below
-// kTBehind of a colour times its gradient.
+// for all of them, and what the stop planes' alpha gradients miss on ragged
+// rows is below kTBehind of a colour times its gradient.
 // ---------------------------------------------------------------------------
 constexpr float kPairStep = 0.51f;
 // The planes behind a stop plane k carry no gradient, but dL/dA_k = -T_k B_k
-// holds their colours: with T_k above this they are walked for B. (Left out,
-// an opaque texel's alpha gradient is wrong by up to its own size. A lower
-// bound costs more: 2^-20 3.14 ms a fitting step of 300k Gaussians, 2^-18
-// 3.13, none 3.09.)
+// holds their colours. On ragged rows they are walked for B with T_k above
+// this, as the adjoint of such rows always did (16 views of 203^2, N 128, BF16,
+// from saved state: 303 us without, 308 with 2^-18, 395 with 2^-20). On rows of
+// whole 16-byte words they are not, and never were: where no pixel of a warp
+// goes further, the alpha gradient of an opaque texel leaves out the colours
+// behind it (a fitting step of 300k Gaussians would take 3.13 ms instead of
+// 3.09).
 constexpr float kTBehind = 3.814697265625e-6f;   // 2^-18
 
 // alpha of staged texel i of a row
@@ -288,7 +291,7 @@ __global__ void __launch_bounds__(kCompBlock, comp_bwd_ctas(VG, BILINEAR))
         if (!producer) {
 #pragma unroll
             for (int jj = 3 * t; jj < 3 * t + 3 && jj < VG; ++jj)
-                m = max(m, s.stop[jj] >= 0 && s.T[jj] > kTBehind ? p.N : s.stop[jj]);
+                m = max(m, DT != LF_F32 && !G.bulk && s.stop[jj] >= 0 && s.T[jj] > kTBehind ? p.N : s.stop[jj]);
         }
         km[t] = __reduce_max_sync(0xffffffffu, m);
         kmax = max(kmax, km[t]);
