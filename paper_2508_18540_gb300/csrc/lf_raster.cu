@@ -240,10 +240,18 @@ __device__ __forceinline__ void raster_gauss_list(const BuildWs& w, const Raster
         const ulonglong2* s_e1 = sm.e1[buf];
         const ulonglong2* s_e2 = sm.e2[buf];
         const float4* s_e3 = sm.e3[buf];
+        // 3DGS: a block whose pixels have all stopped is done (1.4M Gaussians on 21
+        // planes of 1230 x 812, most pixels stopped: 3.79 -> 2.15 ms; tested for
+        // every 32 entries 1.80, but 1 % slower where few pixels stop)
+        uint32_t on_upper = 1u, on_lower = 1u;
+        if (G3 && base > 0) {
+            on_upper = __all_sync(0xffffffffu, (stopped & 0x0011u) == 0x0011u) ? 0u : 1u;
+            on_lower = __all_sync(0xffffffffu, (stopped & 0x1100u) == 0x1100u) ? 0u : 1u;
+        }
         for (int m0 = 0; m0 < cnt; m0 += 32) {
             const uint32_t wm = m0 + lane < cnt ? sm.wm[buf][m0 + lane] : 0u;
-            const uint32_t upper = __ballot_sync(0xffffffffu, (wm >> warp) & 1u);
-            const uint32_t lower = __ballot_sync(0xffffffffu, (wm >> (8 + warp)) & 1u);
+            const uint32_t upper = __ballot_sync(0xffffffffu, (wm >> warp) & on_upper);
+            const uint32_t lower = __ballot_sync(0xffffffffu, (wm >> (8 + warp)) & on_lower);
             auto walk = [&](auto finite) {
                 uint32_t mask = upper | lower;
                 while (mask) {
