@@ -275,18 +275,19 @@ lf_status lf_composite_status(int32_t N, const lf_view_set* views, const void* c
 
 /* Allocation-free form of lf_composite (the paper has no counterpart): the
  * same kernels and the same result, with the composite scratch (coefficient
- * tables and the error word) in a static device array of
- * lf_composite_noalloc_max_bytes() bytes (1 MiB) inside the library instead
- * of a caller workspace. It is for callers that cannot hand the library device
+ * tables and the error word) in a static device array inside the library
+ * (lf_composite_noalloc_max_bytes() bytes, 1 MiB, and 4 KiB for the tables'
+ * alignment) instead of a caller workspace. It is for callers that cannot hand the library device
  * memory, for example a display runtime's per-frame present callback, which
  * runs where calling a device allocator is not allowed (it may synchronise
  * the device or stall the frame). Every GPU that loads the library holds the
  * array until the process exits. Each call looks up the array's device
  * address on the calling thread's current device (cudaGetSymbolAddress, no
  * allocation); the first call on a device may load the library's device code
- * there, so make it before any stream capture. Requests whose scratch
- * (lf_composite_workspace_size) exceeds the limit fail with LF_ERR_WORKSPACE
- * and a message, before any device work. Every call shares the one array and
+ * there, so make it before any stream capture. Requests for which
+ * 12 Vx N + 12 Vy N + 4 N bytes (the tables of one view per group, each term
+ * rounded up to 256) exceed the limit fail with LF_ERR_WORKSPACE and a
+ * message, before any device work. Every call shares the one array and
  * it keeps the last call's contents (the error word is cleared by each
  * call): calls that overlap on the GPU race, so the caller must serialise
  * them. A bounded device wait that gives up is reported by
@@ -451,7 +452,7 @@ typedef struct lf_batch lf_batch;   /* opaque host-side batch object */
 lf_status lf_batch_create(const lf_batch_scene* scenes, int32_t n_scenes, lf_batch** out);
 
 /* Device bytes of the batch workspace for plans with one chunk group (scene
- * tables and work counters). */
+ * tables). */
 size_t lf_batch_workspace_size(const lf_batch* b);
 
 /* Device bytes of the batch workspace for plan (NULL = default): the tables
@@ -462,7 +463,9 @@ size_t lf_batch_plan_workspace_size(const lf_batch* b, const lf_batch_plan* plan
 /* Sets the plan (NULL = default {9, 512, 1, 1}) and uploads the scene tables
  * into ws (device, ws_bytes >= lf_batch_plan_workspace_size, 256-byte
  * aligned) on stream. Must be called before lf_batch_render and again after
- * a plan change; not during capture. */
+ * a plan change; not during capture. Schedules 0 and 1 take batches for which
+ * six stages of whole plane rows and a table of the largest N would fit 200 KB
+ * (LF_ERR_UNSUPPORTED otherwise; schedule 2 takes any). */
 lf_status lf_batch_prepare(lf_batch* b, const lf_batch_plan* plan, void* ws, size_t ws_bytes, cudaStream_t stream);
 
 /* Enqueues one frame of the whole batch on stream (builds, raster,

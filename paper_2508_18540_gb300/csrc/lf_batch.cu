@@ -47,7 +47,7 @@ size_t align256(size_t v) { return (v + 255) / 256 * 256; }
 
 size_t batch_tables_bytes(int n)
 {
-    return align256(16) + align256(sizeof(RasterScene) * n) + align256(sizeof(CompScene) * n);
+    return align256(sizeof(RasterScene) * n) + align256(sizeof(CompScene) * n);
 }
 
 // bytes of one scene's chunk-group partials (groups 1 .. groups - 1)
@@ -74,8 +74,9 @@ bool plan_valid(const lf_batch_plan& pl)
 }
 
 // Size limit of schedules 0 and 1: six stages of whole plane rows of a
-// tile_x x (256 / tile_x) tile and a table of maxN planes fit 200 KB. (The
-// composite itself stages only the windows that its tiles sample.)
+// tile_x x (256 / tile_x) tile and a table of maxN planes fit 200 KB. It is the
+// batches' contract, not a need of the composite, which stages only the windows
+// that its tiles sample.
 size_t batch_row_bytes(const CompParams& p, int tb, int tile_x)
 {
     const int tx = std::min({(p.Nx + 31) / 32 * 32, tile_x, 256});
@@ -162,8 +163,8 @@ lf_status lf_batch_prepare(lf_batch* b, const lf_batch_plan* plan, void* ws, siz
     if (ws_bytes < batch_ws_bytes(b, groups))
         return fail(LF_ERR_WORKSPACE, "batch workspace too small for this plan (lf_batch_plan_workspace_size)");
     char* base = static_cast<char*>(ws);
-    b->rtab = reinterpret_cast<RasterScene*>(base + align256(16));
-    b->ctab = reinterpret_cast<CompScene*>(base + align256(16) + align256(sizeof(RasterScene) * n));
+    b->rtab = reinterpret_cast<RasterScene*>(base);
+    b->ctab = reinterpret_cast<CompScene*>(base + align256(sizeof(RasterScene) * n));
 
     const int tb = texel_bytes(b->dtype);
     std::vector<RasterScene> r(n);
@@ -207,8 +208,8 @@ lf_status lf_batch_prepare(lf_batch* b, const lf_batch_plan* plan, void* ws, siz
         tab_rows = std::max(tab_rows, rows);
     }
     if (pl.schedule != 2 && 6 * row_bytes + batch_table_bytes(maxN, pl.views_per_thread) > 200 * 1024)
-        return fail(LF_ERR_UNSUPPORTED, "lf_batch_prepare: the batch's largest plane row and N need more than "
-                                        "200 KB of shared memory for the staged composite");
+        return fail(LF_ERR_UNSUPPORTED, "lf_batch_prepare: the batch's largest plane row and N are past the limit of "
+                                        "schedules 0 and 1 (six stages of whole rows and the table within 200 KB)");
     // schedule: order of the scenes in the item tables
     std::vector<int> ro(n), co(n);
     for (int i = 0; i < n; ++i) ro[i] = co[i] = i;

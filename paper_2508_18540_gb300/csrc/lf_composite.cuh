@@ -937,8 +937,9 @@ __device__ __forceinline__ void composite_tile(const CompParams& p, const CompGe
 // launch's own size would refuse a larger launch of another thread.
 constexpr size_t kCompSmemMax = 200 * 1024;
 
-// CTAs per SM that the adjoint's registers leave room for: nearest, bound by
-// its atomics, 9 views at 96 registers, 3 at 64; bilinear 9 at 128 and 3 at 96,
+// CTAs per SM that the adjoint's registers leave room for: nearest 9 views at 96
+// registers and 3 at 64 (9 at 128: 3.22 ms a fitting step of 300k Gaussians
+// instead of 3.10, with fewer spills but fewer warps); bilinear 9 at 128 and 3 at 96,
 // without spills (fitting steps of 256^2, N 64, 12 views: 1.32 ms with 96 and
 // 64, 0.95 now; 45 views 2.72 and 2.29).
 __host__ __device__ constexpr int comp_bwd_ctas(int VG, bool bilinear)

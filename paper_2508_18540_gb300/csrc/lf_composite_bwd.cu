@@ -22,12 +22,14 @@ namespace {
 // it, at most four planes earlier, each leaving at least 2^-24).
 //
 // The forward's staged tiles are used (4 consumer warps, windows of plane
-// rows in the ring). Nearest: bound by the rate of 16-byte atomics to L2
-// (one per sample: 1.77 ms on 45 views of 512^2, N 64, with 35 % fewer
-// instructions than a kernel that took 1.72), so a thread adds up the
-// gradients of consecutive views while they sample the same texel (neighbouring
-// views shift by under a texel near the focal plane) and adds a run to
-// dplanes with one FP32 vector atomic. Three views' texels are loaded before
+// rows in the ring). Nearest: a 16-byte atomic per sample cost more than its
+// instructions (1.77 ms on 45 views of 512^2, N 64, with 35 % fewer instructions
+// than a kernel that took 1.72), so a thread adds up the gradients of
+// consecutive views while they sample the same texel (neighbouring views shift
+// by under a texel near the focal plane) and adds a run to dplanes with one FP32
+// vector atomic. With the runs no unit is the bound alone (from saved state, FP32:
+// issue slots 61 % busy, requests from L1 to L2 54 %, L2's atomic units 32 %, DRAM
+// 9 %, at 18 warps per SM). Three views' texels are loaded before
 // their steps back, so that the loads overlap. (Summing a plane's gradients
 // per warp in shared memory first takes 12 to 16 shared-memory wavefronts a
 // sample, where the texel and the atomic take 8: 1.72 ms.)

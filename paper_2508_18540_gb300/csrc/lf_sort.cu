@@ -21,8 +21,10 @@
 //    (super-tile, rank) pair emitted in rank order; the stable sort groups the
 //    pairs by super-tile and keeps each one's pairs in depth order.
 //
-// One kernel per pass (k_sweep), with the digit totals of all passes known
-// beforehand (k_depth_hist; the pair emission): a block of 512 threads ranks
+// One kernel per pass (k_sweep), by decoupled look-back (Merrill and Garland,
+// Single-pass Parallel Prefix Scan with Decoupled Look-back, 2016), with the
+// digit totals of all passes known beforehand (k_depth_hist; the pair
+// emission): a block of 512 threads ranks
 // its 2048 or 4096 keys stably (ballot-based digit matching, per-warp
 // counters, warps own contiguous key ranges), publishes its digit counts,
 // exchanges the keys through shared memory into digit order, adds up the
