@@ -69,7 +69,6 @@ constexpr int kEmitStage = 4096;   // pairs
 // atomic per pair on four words serialises (with the staging above: 48 -> 25 us
 // for 5M pairs on 1024 super-tiles; with fewer pairs the folding costs more).
 constexpr int kFoldSupers = 1024;
-constexpr uint32_t kNoBlock = 0xffffffffu;   // no place among the blocks: a wait gave up
 
 // Chunks and copies (BIN) and pairs (EMIT) of PER ranks per thread, kT apart.
 // One kernel does both for few primitives, where launches and latencies
@@ -100,15 +99,16 @@ __global__ void __launch_bounds__(kT, EMIT ? 4 : 6) k_bin_emit(BuildWs w, BinPar
         // After a wait gave up (of the sort, or in an earlier block here) valA is
         // no order: no block does anything. (Depths out of order give bins below
         // zero, and chunk_start would be written there.)
-        const uint32_t place = !EMIT ? blockIdx.x : atomicAdd(&w.hdr->ticket[kDepthPasses + kTilePassesMax], 1u);
-        const bool disparity = BIN && p.binning != LF_BIN_QUANTILE && M > 0;
-        const uint32_t first = disparity ? w.valA[0] : 0u, last = disparity ? w.valA[M - 1] : 0u;   // beside the flag's load
-        const bool valid = !w.hdr->timeout;
-        s_block = valid ? place : kNoBlock;
-        if (disparity && valid) {
+        s_block = EMIT ? atomicAdd(&w.hdr->ticket[kDepthPasses + kTilePassesMax], 1u)
+                       : w.hdr->timeout ? kNoTicket : blockIdx.x;
+        if (BIN && p.binning != LF_BIN_QUANTILE && M > 0) {
+            // (read in bounds without waiting for the ticket, in order or not)
+            const uint32_t last_prim = (uint32_t)(w.hdr->n - 1);
+            const double zmin = __longlong_as_double((long long)w.keyA[min(w.valA[0], last_prim)]);
+            const double zmax = __longlong_as_double((long long)w.keyA[min(w.valA[M - 1], last_prim)]);
             DispRange d;
-            d.izmin = __ddiv_rn(1.0, __longlong_as_double((long long)w.keyA[first]));
-            d.span = __dsub_rn(d.izmin, __ddiv_rn(1.0, __longlong_as_double((long long)w.keyA[last])));
+            d.izmin = __ddiv_rn(1.0, zmin);
+            d.span = __dsub_rn(d.izmin, __ddiv_rn(1.0, zmax));
             d.izminf = __double2float_rn(d.izmin);
             d.scale = (float)p.N / __double2float_rn(d.span);
             d.margin = 4.76837158e-7f * (d.scale * d.izminf + 2.0f * (float)p.N);   // 2^-21
@@ -123,7 +123,7 @@ __global__ void __launch_bounds__(kT, EMIT ? 4 : 6) k_bin_emit(BuildWs w, BinPar
     }
     __syncthreads();
     const long long b = s_block, r0 = b * (PER * kT);
-    if (s_block == kNoBlock) return;
+    if (s_block >= kNoTicket) return;
     if (M == 0) {
         if (BIN && b == 0)
             for (int k = tid; k <= p.N; k += kT) w.chunk_start[k] = 0;
@@ -260,7 +260,7 @@ __global__ void __launch_bounds__(kT, EMIT ? 4 : 6) k_bin_emit(BuildWs w, BinPar
             t -= use;
             idle = use ? 0 : idle + 1;
             if (idle > w.look_tries) {
-                if (lane == 0) atomicExch(&w.hdr->timeout, 1);
+                if (lane == 0) give_up(w.hdr);
                 done = true;
             }
         }

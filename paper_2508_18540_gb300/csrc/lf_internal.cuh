@@ -153,8 +153,8 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity)
 // BuildWs::look_tries times without progress sets WsHeader::timeout and goes on
 // with the sum it has. That sum is never above the true one, so its own writes
 // stay in range, but the order it leaves is not valid: entries are lost, and the
-// places they would have taken hold whatever was there before. So every later
-// kernel of the build and the adjoints start by looking at the flag.
+// places they would have taken hold whatever was there before. So no later
+// block of the build works on it, nor do the adjoints (give_up, no_lists).
 #ifdef __CUDACC__
 constexpr unsigned long long kSumOwn = 1ull << 62, kSumAll = 2ull << 62, kSumMask = kSumOwn - 1ull;
 constexpr int kLookbackTries = 1 << 20;   // polls without progress (about a second) before a block gives up
@@ -262,10 +262,11 @@ struct WsHeader {
     unsigned long long kmin;      // smallest / largest valid depth key
     unsigned long long kmax;
     unsigned long long M;         // culled-in primitives
+    int overflow;                 // 1 if total_dups > dup_capacity
+    int timeout;                  // a bounded wait of the build gave up (read beside M)
     unsigned long long total_dups;
     unsigned long long tile_n;    // pairs to sort (0 after an overflow)
     unsigned long long long_runs; // depth-sort runs longer than 32 keys, sorted by k_depth_long_runs
-    int overflow;                 // 1 if total_dups > dup_capacity
     int kind;                     // 0 gaussians, 1 voxels
     long long n;
     long long dup_capacity;
@@ -278,11 +279,19 @@ struct WsHeader {
     // blocks of the sweeps and of the binning take their place in order from
     // these counters, so that a block only ever waits for running ones
     unsigned int ticket[kDepthPasses + kTilePassesMax + 1];
-    int timeout;                  // a bounded wait of the build gave up
 };
 
-// The build made no lists, and its order may be none: the adjoints give zero gradients.
+// A wait gave up: the flag for the host and the kernels without tickets, and no
+// more tickets, so that the blocks that take one need not look at the flag.
+constexpr unsigned int kNoTicket = 1u << 31;
 #ifdef __CUDACC__
+__device__ __forceinline__ void give_up(WsHeader* h)
+{
+    atomicExch(&h->timeout, 1);
+    for (unsigned int& t : h->ticket) atomicMax(&t, kNoTicket);
+}
+
+// The build made no lists, and its order may be none: the adjoints give zero gradients.
 __device__ __forceinline__ bool no_lists(const WsHeader& h) { return h.overflow || h.timeout; }
 #endif
 

@@ -163,13 +163,11 @@ __global__ void __launch_bounds__(kSweepThreads, 2) k_sweep(const void* __restri
     SweepSmem<KPT>& S = *reinterpret_cast<SweepSmem<KPT>*>(sweep_raw);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const long long n = a.n_dev ? (long long)*a.n_dev : a.n_static;
-    if (tid == 0) {
-        // After a wait gave up (in a pass before, or in an earlier block of this
-        // one) no block does anything: the keys may hold stale ones, which the
-        // digit totals don't count, and their places could lie past the arrays.
-        const uint32_t place = atomicAdd(&a.hdr->ticket[a.pass], 1u);
-        S.tile = a.hdr->timeout ? 0xffffffffu : place;   // past any count of keys
-    }
+    // After a wait gave up (in a pass before, or in an earlier block of this one)
+    // no block does anything: the tickets lie past any count of keys. (The keys
+    // may hold stale ones then, which the digit totals don't count, and their
+    // places could lie past the arrays.)
+    if (tid == 0) S.tile = atomicAdd(&a.hdr->ticket[a.pass], 1u);
     for (int i = tid; i < kWarps * kDigits; i += kSweepThreads) (&S.wcnt[0][0])[i] = 0u;
     __syncthreads();
     const long long tile = S.tile, blk = tile * (kSweepThreads * KPT);
@@ -259,7 +257,7 @@ __global__ void __launch_bounds__(kSweepThreads, 2) k_sweep(const void* __restri
             t -= u;
             idle = u ? 0 : idle + 1;
             if (idle > a.look_tries) {
-                atomicExch(&a.hdr->timeout, 1);
+                give_up(a.hdr);
                 done = true;
             }
         }
